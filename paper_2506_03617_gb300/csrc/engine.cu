@@ -95,7 +95,9 @@ struct mxp_problem {
     double *c_dev = nullptr;
     double *kappa64 = nullptr;
     float *kappa32 = nullptr;
-    double2 *coef64 = nullptr;
+    double2 *coef64 = nullptr;            // coefficient table times h^2
+    double2 *diag64 = nullptr;            // scaled diagonal of the complex128 actions (ensure_diag)
+    bool diag_ok = false;                 // diag64 belongs to the current parameters and faces
     float2 *coef32 = nullptr;
     float2 *coef32s = nullptr;           // coef32 scaled by h^2 in double (persistent kernel)
     // ghost-point faces (mxp_set_boundary): condition per face, and the diagonal
@@ -321,7 +323,10 @@ static mxp_status upload_coefs(mxp_problem *P)
 {
     build_coef_host(P);
     const size_t cnt = P->coef_host.size();
-    CK(cudaMemcpyAsync(P->coef64, P->coef_host.data(), cnt * sizeof(double2), cudaMemcpyHostToDevice, P->stream));
+    const double h2 = P->grid.h * P->grid.h;
+    std::vector<double2> c64(cnt);
+    for (size_t i = 0; i < cnt; ++i) c64[i] = make_double2(P->coef_host[i].x * h2, P->coef_host[i].y * h2);
+    CK(cudaMemcpyAsync(P->coef64, c64.data(), cnt * sizeof(double2), cudaMemcpyHostToDevice, P->stream));
     compute_kappa(P->c_dev, P->prm.omega, P->kappa64, P->kappa32, P->ntot, P->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(P->stream));
@@ -379,9 +384,12 @@ static mxp_status ensure_arnoldi(mxp_problem *P, Arnoldi &a, int R, bool flexibl
     return MXP_OK;
 }
 
+static mxp_status ensure_diag(mxp_problem *P);
+
 static mxp_status ensure_base(mxp_problem *P)
 {
     const int64_t n = P->ntot;
+    if (P->prm.prec == MXP_C128) CKS(ensure_diag(P));
     for (int i = 0; i < 4; ++i)
         if (!P->hb[i]) CK(cudaMalloc(&P->hb[i], (size_t)n * 16));
     if (!P->rt) CK(cudaMalloc(&P->rt, n * sizeof(double2)));
@@ -440,6 +448,35 @@ static void set_faces(const mxp_problem *P, StepScalars<typename St<S>::C> &sc)
         sc.face[f] = (P->bc[f] != MXP_BC_DIRICHLET) ? PrecData<S>::faces(P) + P->face_off[f] : nullptr;
 }
 template <> struct PrecData<__nv_bfloat162> : PrecData<float2> {};
+
+// The scaled diagonal of the complex128 actions: made before the first action
+// after a change of parameters or faces (a slab's at its set-up: mxp_horner_step
+// neither allocates nor launches more than its sweep).
+static mxp_status ensure_diag(mxp_problem *P)
+{
+    if (P->diag_ok) return MXP_OK;
+    if (!P->diag64) CK(cudaMalloc(&P->diag64, (size_t)P->ntot * sizeof(double2)));
+    StepScalars<double2> sc{};
+    sc.zfac = make_double2(1.0, P->prm.shift_s);
+    sc.mu = P->mu;
+    set_faces<double2>(P, sc);
+    make_diag64(P->geom, P->coef64, P->kappa64, sc, P->diag64, P->stream);
+    CK(cudaGetLastError());
+    P->diag_ok = true;
+    return MXP_OK;
+}
+
+// One Taylor-Horner sweep of an action.  chain: it follows another sweep of the
+// same sequence on st.
+template <typename S>
+static void sweep(mxp_problem *P, const StepScalars<typename St<S>::C> &sc, const S *pin, const S *y, const S *v,
+                  S *pout, cudaStream_t st, bool chain)
+{
+    if constexpr (sizeof(S) == sizeof(double2))
+        launch_step64(P->geom, P->coef64, P->kappa64, P->diag64, sc, pin, y, v, pout, st, chain);
+    else
+        launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc, pin, y, v, pout, st);
+}
 
 template <typename S>
 static bool fused_pass(mxp_problem *P, int cfg, const FusedStep *steps, const S *pin, const S *y,
@@ -888,7 +925,7 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
             sc.gamma = PrecData<S>::c(augq.gamma(k));
             sc.rho = PrecData<S>::c(cd(1.0));
             const int o = (in == 0) ? 1 : 3 - in;           // y = b[0] (zero) throughout
-            launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc, b[in], b[0], vs, b[o], st);
+            sweep<S>(P, sc, b[in], b[0], vs, b[o], st, in != 0);
             augq.step(k);
             in = o;
         }
@@ -980,9 +1017,7 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
                     done = true;
                 }
             }
-            if (!done)
-                launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc, b[in], b[iy],
-                               which ? vs : nullptr, b[o], st);
+            if (!done) sweep<S>(P, sc, b[in], b[iy], which ? vs : nullptr, b[o], st, passes > 0);
             aug.step(k);
             in = o;
             ++passes;
@@ -1013,7 +1048,7 @@ static void apply_op(mxp_problem *P, int shifted, const double2 *x, double2 *y, 
     sc.gamma = make_double2(0.0, 0.0);
     sc.rho = make_double2(1.0, 0.0);
     set_faces<double2>(P, sc);
-    launch_step<double2>(P->geom, P->coef64, P->kappa64, sc, x, nullptr, nullptr, y, st ? st : P->stream);
+    launch_step64(P->geom, P->coef64, P->kappa64, nullptr, sc, x, nullptr, nullptr, y, st ? st : P->stream, false);
     P->passes += 1;
 }
 
@@ -1351,8 +1386,8 @@ static int batch_sweeps(mxp_problem *P, int which, int nb, const TaylorPlan &pl,
                 sc.gamma = PrecData<S>::c(aug.gamma(k));
                 sc.rho = PrecData<S>::c((sub == Ssub - 1 && k == 1) ? final_rho : cd(1.0));
                 for (int j = 0; j < nb; ++j)
-                    launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc, b[in] + j * n,
-                                   b[iy] + j * n, vs ? vs + j * n : nullptr, b[o] + j * n, st);
+                    sweep<S>(P, sc, b[in] + j * n, b[iy] + j * n, vs ? vs + j * n : nullptr, b[o] + j * n, st,
+                             *passes > 0 || j > 0);
                 aug.step(k);
             }
             in = o;
@@ -2186,6 +2221,11 @@ static mxp_status create_impl(const mxp_grid *grid, int64_t row0, int64_t nrows,
     P->geom.fast = slab ? 0 : 1;
     P->geom.npml = grid->npml;
     P->geom.ih2 = 1.0 / (grid->h * grid->h);
+    for (int d = 0; d < 3; ++d) {
+        const int off = (slab && d == grid->dim - 1) ? (int)row0 : 0;
+        P->geom.in_lo[d] = d < grid->dim ? grid->npml - off : 0;
+        P->geom.in_hi[d] = d < grid->dim ? (int)(grid->n_interior[d] + grid->npml) - off : 1;
+    }
     P->ntot = ntot;
     P->cmin = cmin;
     P->cmax = cmax;
@@ -2205,6 +2245,7 @@ static mxp_status create_impl(const mxp_grid *grid, int64_t row0, int64_t nrows,
     if (s != MXP_OK) return bail(s);
     update_plans(P);
     s = upload_coef32(P);
+    if (s == MXP_OK && slab) s = ensure_diag(P);
     if (s == MXP_OK) s = retune(P);
     if (s != MXP_OK) return bail(s);
     *out = P;
@@ -2238,8 +2279,8 @@ mxp_status mxp_horner_step(mxp_problem *P, const double *sigma, const double *ga
     sc.gamma = v_dev ? make_double2(gamma[0], gamma[1]) : make_double2(0.0, 0.0);
     sc.rho = make_double2(rho[0], rho[1]);
     set_faces<double2>(P, sc);
-    launch_step<double2>(P->geom, P->coef64, P->kappa64, sc, (const double2 *)p_dev, (const double2 *)y_dev,
-                         (const double2 *)v_dev, (double2 *)out_dev, P->stream);
+    launch_step64(P->geom, P->coef64, P->kappa64, P->diag_ok ? P->diag64 : nullptr, sc, (const double2 *)p_dev,
+                  (const double2 *)y_dev, (const double2 *)v_dev, (double2 *)out_dev, P->stream, false);
     P->passes += 1;
     CK(cudaGetLastError());
     return MXP_OK;
@@ -2392,6 +2433,7 @@ mxp_status mxp_set_boundary(mxp_problem *P, const int *bc)
     }
     P->nfaces = nf;
     CKS(build_faces(P));
+    P->diag_ok = false;
     clear_graphs(P);
     return retune(P);
 }
@@ -2431,6 +2473,8 @@ mxp_status mxp_set_params(mxp_problem *P, const mxp_params *p)
     if (recoef && P->nfaces) CKS(build_faces(P));
     update_plans(P);
     CKS(upload_coef32(P));
+    P->diag_ok = false;
+    if (P->slab) CKS(ensure_diag(P));
     clear_graphs(P);
     return retune(P);
 }
@@ -2720,7 +2764,7 @@ void mxp_destroy(mxp_problem *P)
     DeviceGuard guard(P->device);
     cudaStreamSynchronize(P->stream);
     cudaFree(P->c_dev); cudaFree(P->kappa64); cudaFree(P->kappa32);
-    cudaFree(P->coef64); cudaFree(P->coef32); cudaFree(P->coef32s);
+    cudaFree(P->coef64); cudaFree(P->diag64); cudaFree(P->coef32); cudaFree(P->coef32s);
     cudaFree(P->face64); cudaFree(P->face32); cudaFree(P->face32s);
     for (int i = 0; i < 4; ++i) cudaFree(P->hb[i]);
     tma3_destroy(P->tma3);

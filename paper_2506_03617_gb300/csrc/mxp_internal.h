@@ -96,6 +96,9 @@ struct Geom {
     int fast = 0;      // 1: unknowns outside the PML use the real interior coefficient ih2
     int npml = 0;
     double ih2 = 0;    // 1 / h^2
+    // positions [in_lo, in_hi) of each axis lie outside its PML: their neighbour
+    // coefficients are the real 1 / h^2 (complex128 sweeps)
+    int in_lo[3] = {0, 0, 0}, in_hi[3] = {1, 1, 1};
 };
 
 // Scalars of one Taylor-Horner step  out = rho * (y + sigma * (A_s - mu) p + gamma * v)
@@ -135,6 +138,17 @@ template <typename S>
 void launch_step(const Geom &g, const typename St<S>::C *coef, const typename St<S>::R *kappa,
                  const StepScalars<typename St<S>::C> &sc, const S *pin, const S *y, const S *v,
                  S *pout, cudaStream_t st);
+
+// The same step in complex128 (stencil64.cu); coef is the table times h^2.  diag
+// (nullable): the sweep's scaled diagonal from make_diag64, formed per point
+// otherwise.  chain: the launch may start before the launch preceding it on st
+// has ended; only where that one is a complex128 sweep too.
+void launch_step64(const Geom &g, const double2 *coef, const double *kappa, const double2 *diag,
+                   const StepScalars<double2> &sc, const double2 *pin, const double2 *y, const double2 *v,
+                   double2 *pout, cudaStream_t st, bool chain);
+// diag = h^2 (kappa zfac - mu - sum_d wc_d + face terms) of every unknown, for sc's zfac, mu and faces.
+void make_diag64(const Geom &g, const double2 *coef, const double *kappa, const StepScalars<double2> &sc,
+                 double2 *diag, cudaStream_t st);
 
 // Fused passes (2D): K consecutive Horner steps of one sub-step per launch,
 // tiled through shared memory with a K-cell halo.  Step s uses

@@ -73,11 +73,11 @@ struct AxisGeom {
     double L[3];
 };
 
+// The table times h^2, as the complex128 sweep takes it.
 __global__ void k_noalloc_coef(AxisGeom ag, int dim, int npml, double h, double cpml, double omega,
                                int nmax)
 {
     double2 *coef = reinterpret_cast<double2 *>(g_noalloc_scratch + kCoefOff);
-    const double ih2 = 1.0 / (h * h);
     for (int d = 0; d < dim; ++d) {
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ag.n[d]; i += gridDim.x * blockDim.x) {
             const double x = ((double)i - npml + 0.5) * h;
@@ -85,8 +85,8 @@ __global__ void k_noalloc_coef(AxisGeom ag, int dim, int npml, double h, double 
             inv_stretch_nd(x, ag.L[d], npml, h, cpml, omega, &ar, &ai);
             inv_stretch_nd(x + 0.5 * h, ag.L[d], npml, h, cpml, omega, &pr, &pi);
             inv_stretch_nd(x - 0.5 * h, ag.L[d], npml, h, cpml, omega, &mr, &mi);
-            const double2 wp = make_double2((ar * pr - ai * pi) * ih2, (ar * pi + ai * pr) * ih2);
-            const double2 wm = make_double2((ar * mr - ai * mi) * ih2, (ar * mi + ai * mr) * ih2);
+            const double2 wp = make_double2(ar * pr - ai * pi, ar * pi + ai * pr);
+            const double2 wm = make_double2(ar * mr - ai * mi, ar * mi + ai * mr);
             coef[(size_t)(3 * d + 0) * nmax + i] = wp;
             coef[(size_t)(3 * d + 1) * nmax + i] = wm;
             coef[(size_t)(3 * d + 2) * nmax + i] = make_double2(wp.x + wm.x, wp.y + wm.y);
@@ -231,6 +231,12 @@ extern "C" mxp_status mxp_apply_phi_noalloc(const mxp_grid *grid, const mxp_para
     g.s2 = (int64_t)ag.n[0] * ag.n[1];
     g.ntot = ntot;
     g.nmax = nmax;
+    g.npml = grid->npml;
+    g.ih2 = 1.0 / (grid->h * grid->h);
+    for (int d = 0; d < grid->dim; ++d) {
+        g.in_lo[d] = grid->npml;
+        g.in_hi[d] = ag.n[d] - grid->npml;
+    }
     const size_t bytes = (size_t)ntot * sizeof(double2);
     const double2 *v = nullptr;
     if (which == 0) {
@@ -259,7 +265,7 @@ extern "C" mxp_status mxp_apply_phi_noalloc(const mxp_grid *grid, const mxp_para
             const cd rho = (sub == Sbest - 1 && k == 1) ? final_rho : cd(1.0);
             sc.rho = make_double2(rho.real(), rho.imag());
             const int o = (in == iy) ? (iy + 1) % 3 : 3 - iy - in;
-            launch_step<double2>(g, coef, kappa, sc, buf[in], buf[iy], v, buf[o], st);
+            launch_step64(g, coef, kappa, nullptr, sc, buf[in], buf[iy], v, buf[o], st, passes > 0);
             pxi = yxi + rot * pxi / (double)k;
             in = o;
             ++passes;

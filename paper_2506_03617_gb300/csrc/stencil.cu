@@ -1,6 +1,6 @@
-// Stencil kernels: the PML Helmholtz operator and one Taylor-Horner step of the
-// exponential-integrator actions (Def. psi), for complex128, complex64 and
-// bfloat16-storage vectors.
+// Stencil kernels: one Taylor-Horner step of the exponential-integrator actions
+// (Def. psi) for complex64 and bfloat16-storage vectors (complex128: stencil64.cu),
+// and the conversions between the stored types.
 //
 // Operator (Eq. helmholtz with the stretched Laplacian of Eq. pml-1d-s on each
 // axis, shift of Sec. 3.4), written with the per-axis coefficient table
@@ -216,13 +216,8 @@ void launch_step(const Geom &g, const typename St<S>::C *coef, const typename St
                  const StepScalars<typename St<S>::C> &sc, const S *pin, const S *y, const S *v,
                  S *pout, cudaStream_t st)
 {
-    if constexpr (sizeof(S) <= 8) {                                      // complex64 / bf16 storage
-        if (g.dim == 3 && sc.nfaces == 0) {
-            launch_step3z<S>(g, coef, kappa, sc, pin, y, v, pout, st);
-            return;
-        }
-    }
-    if (g.dim == 3) launch_step_dim<S, 3>(g, coef, kappa, sc, pin, y, v, pout, st);
+    if (g.dim == 3 && sc.nfaces == 0) launch_step3z<S>(g, coef, kappa, sc, pin, y, v, pout, st);
+    else if (g.dim == 3) launch_step_dim<S, 3>(g, coef, kappa, sc, pin, y, v, pout, st);
     else launch_step_dim<S, 2>(g, coef, kappa, sc, pin, y, v, pout, st);
 }
 
@@ -271,16 +266,20 @@ void launch_convert_out(const S *x, double2 *out, const double2 *base, int mode,
     k_convert_out<S><<<stream_grid(n), 256, 0, st>>>(x, out, base, mode, n);
 }
 
-#define MXP_INST(S)                                                                          \
+#define MXP_INST_STEP(S)                                                                     \
     template void launch_step<S>(const Geom &, const St<S>::C *, const St<S>::R *,           \
                                  const StepScalars<St<S>::C> &, const S *, const S *,        \
-                                 const S *, S *, cudaStream_t);                              \
+                                 const S *, S *, cudaStream_t);
+#define MXP_INST(S)                                                                          \
     template void launch_convert_in<S>(const double2 *, S *, int64_t, cudaStream_t);         \
     template void launch_convert_out<S>(const S *, double2 *, const double2 *, int, int64_t, \
                                         cudaStream_t);
 MXP_INST(double2)
 MXP_INST(float2)
 MXP_INST(__nv_bfloat162)
+MXP_INST_STEP(float2)
+MXP_INST_STEP(__nv_bfloat162)
 #undef MXP_INST
+#undef MXP_INST_STEP
 
 }  // namespace mxp
