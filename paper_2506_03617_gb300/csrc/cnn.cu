@@ -3,9 +3,10 @@
 // Adam kernels (training and inference run on the GPU).  The forward
 // convolutions, the input gradients and the weight gradients run on the tensor
 // cores (tcgen05, bfloat16 operands, float32 accumulation in tensor memory;
-// conv_tc.cu); the bias gradients and the elementwise steps on CUDA cores.  The paper has no
-// learned stage; this is the project's own extension, used as an extra
-// FGMRES stage with MatExPre as fallback (see engine.cu).
+// conv_tile.cu), with the elementwise steps (bias, relu, skip, masks, pooling, bias
+// gradients) inside those kernels.  The paper has no learned stage; this is the
+// project's own extension, used as an extra FGMRES stage with MatExPre as
+// fallback (see engine.cu).
 //
 // Network (NCHW, 3x3 kernels, zero padding 1):
 //   a1 = relu(conv(x, W1) + b1)                 3 -> 32
@@ -39,55 +40,6 @@ static int64_t layer_woff(int l)
 int64_t cnn_num_params() { return layer_woff(6); }
 
 // ---------------------------------------------------------------- backward
-// gb[co] = sum over images and pixels of gout[n, co, :, :]; one block per
-// channel, fixed-order reduction.
-__global__ void __launch_bounds__(256) k_bias_grad(const float *__restrict__ gout, int N, int Cout, int64_t hw,
-                                                   float *__restrict__ gb)
-{
-    const int co = blockIdx.x;
-    float acc = 0.f;
-    for (int n = 0; n < N; ++n) {
-        const float *g = gout + ((int64_t)n * Cout + co) * hw;
-        for (int64_t p = threadIdx.x; p < hw; p += blockDim.x) acc += g[p];
-    }
-    __shared__ float red[8];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float v = 0.f;
-        for (int i = 0; i < 8; ++i) v += red[i];
-        gb[co] = v;
-    }
-}
-
-__global__ void k_relu_mask(float *__restrict__ g, const float *__restrict__ a, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (!(a[i] > 0.f)) g[i] = 0.f;
-}
-
-__global__ void k_add_to(float *__restrict__ a, const float *__restrict__ b, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[i] += b[i];
-}
-
-// g[n, c, i, j] = sum of the 2 x 2 block of gfull (adjoint of nearest upsampling)
-__global__ void k_down2_sum(const float *__restrict__ gfull, int NC, int H, int W, float *__restrict__ g)
-{
-    const int64_t total = (int64_t)NC * H * W;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t nc = i / ((int64_t)H * W);
-        const int r = (int)(i % ((int64_t)H * W));
-        const int y = r / W, x = r % W;
-        const float *b = gfull + nc * 4 * H * W;
-        const int W2 = 2 * W;
-        g[i] = b[(int64_t)(2 * y) * W2 + 2 * x] + b[(int64_t)(2 * y) * W2 + 2 * x + 1] +
-               b[(int64_t)(2 * y + 1) * W2 + 2 * x] + b[(int64_t)(2 * y + 1) * W2 + 2 * x + 1];
-    }
-}
-
 // loss partials and gradient of the mean squared error
 __global__ void k_mse(const float *__restrict__ y, const float *__restrict__ t, int64_t n,
                       float *__restrict__ gy, double *__restrict__ partial)
@@ -177,7 +129,7 @@ struct mxp_cnn {
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *wb = nullptr;
     float *x = nullptr, *a[6] = {nullptr}, *r5 = nullptr, *y = nullptr;
-    float *gy = nullptr, *g5 = nullptr, *gfull = nullptr, *gh = nullptr, *gh2 = nullptr, *g1 = nullptr;
+    float *gy = nullptr, *g5 = nullptr, *gh = nullptr, *gh2 = nullptr, *g1 = nullptr;
     double *partial = nullptr;
     unsigned *err = nullptr;       // set by a tensor-core convolution whose bounded wait gave up
     float *loss_dev = nullptr;
@@ -199,36 +151,36 @@ mxp_status cfail(mxp_status s, const char *m)
                                             cudaGetErrorString(e_));                   \
     } while (0)
 
-template <int S, int UPS>
-void conv_fwd(const mxp_cnn *net, int l, const float *in, int N, int Hs, int Ws, int Ho, int Wo,
-              const float *skip, float *out, float *out_skip)
+// out = act(conv of layer l), out2 (nullable) = out + skip
+bool conv_fwd(const mxp_cnn *net, int l, const float *in, int N, int Hs, int Ws, int Ho, int Wo, const float *skip,
+              float *out, float *out2)
 {
     const CnnLayer L = kNet[l];
     const __nv_bfloat16 *w = net->wb + layer_woff(l);
-    const float *b = net->w + layer_woff(l) + (int64_t)L.cin * L.cout * 9;
-    conv_fwd_tc(S, UPS, in, N, L.cin, Hs, Ws, w, b, L.cout, Ho, Wo, L.relu, skip, out, out_skip, net->err,
-                net->stream);
+    ConvOut o;
+    o.out = out;
+    o.out2 = out2;
+    o.add = skip;
+    return conv_tile(false, L.stride, L.ups, in, N, L.cin, Hs, Ws, w, net->w + layer_woff(l) + (int64_t)L.cin * L.cout * 9,
+                     L.cout, Ho, Wo, L.relu, o, net->err, net->stream);
 }
 
-template <int S>
-void conv_bwd_data(const mxp_cnn *net, int l, const float *gout, int N, int Ho, int Wo, int Hl, int Wl,
-                   float *gin)
+// gradient of layer l's (logical) input, to o
+bool conv_bwd_data(const mxp_cnn *net, int l, const float *gout, int N, int Ho, int Wo, int Hl, int Wl, const ConvOut &o)
 {
     const CnnLayer L = kNet[l];
-    conv_bwd_data_tc(S, gout, N, L.cout, Ho, Wo, net->wb + layer_woff(l), L.cin, Hl, Wl, gin, net->err,
-                     net->stream);
+    return conv_tile(true, L.stride, 0, gout, N, L.cout, Ho, Wo, net->wb + layer_woff(l), nullptr, L.cin, Hl, Wl, 0, o,
+                     net->err, net->stream);
 }
 
-template <int S, int UPS>
-void conv_bwd_weight(const mxp_cnn *net, int l, const float *xin, int N, int Hs, int Ws, const float *gout,
-                     int Ho, int Wo)
+// adds layer l's weight and bias gradients to net->g
+bool conv_bwd_weight(const mxp_cnn *net, int l, const float *xin, int N, int Hs, int Ws, const float *gout, int Ho,
+                     int Wo)
 {
     const CnnLayer L = kNet[l];
     float *gw = net->g + layer_woff(l);
-    float *gb = gw + (int64_t)L.cin * L.cout * 9;
-    conv_wgrad_tc(S, UPS, xin, N, L.cin, Hs, Ws, gout, L.cout, Ho, Wo, gw, net->err, net->stream);
-    count_launch();
-    k_bias_grad<<<L.cout, 256, 0, net->stream>>>(gout, N, L.cout, (int64_t)Ho * Wo, gb);
+    return wgrad_tile(L.stride, L.ups, xin, N, L.cin, Hs, Ws, gout, L.cout, Ho, Wo, gw,
+                      gw + (int64_t)L.cin * L.cout * 9, net->err, net->stream);
 }
 
 mxp_status check_shape(const mxp_cnn *net, int N, int H, int W)
@@ -241,12 +193,13 @@ mxp_status check_shape(const mxp_cnn *net, int N, int H, int W)
 mxp_status forward_impl(mxp_cnn *net, int N, int H, int W, const float *x, float *y)
 {
     const int H2 = H / 2, W2 = W / 2;
-    conv_fwd<1, 0>(net, 0, x, N, H, W, H, W, nullptr, net->a[0], nullptr);
-    conv_fwd<2, 0>(net, 1, net->a[0], N, H, W, H2, W2, nullptr, net->a[1], nullptr);
-    conv_fwd<1, 0>(net, 2, net->a[1], N, H2, W2, H2, W2, nullptr, net->a[2], nullptr);
-    conv_fwd<1, 0>(net, 3, net->a[2], N, H2, W2, H2, W2, nullptr, net->a[3], nullptr);
-    conv_fwd<1, 1>(net, 4, net->a[3], N, H2, W2, H, W, net->a[0], net->r5, net->a[4]);
-    conv_fwd<1, 0>(net, 5, net->a[4], N, H, W, H, W, nullptr, y, nullptr);
+    const bool ok = conv_fwd(net, 0, x, N, H, W, H, W, nullptr, net->a[0], nullptr) &&
+                    conv_fwd(net, 1, net->a[0], N, H, W, H2, W2, nullptr, net->a[1], nullptr) &&
+                    conv_fwd(net, 2, net->a[1], N, H2, W2, H2, W2, nullptr, net->a[2], nullptr) &&
+                    conv_fwd(net, 3, net->a[2], N, H2, W2, H2, W2, nullptr, net->a[3], nullptr) &&
+                    conv_fwd(net, 4, net->a[3], N, H2, W2, H, W, net->a[0], net->r5, net->a[4]) &&
+                    conv_fwd(net, 5, net->a[4], N, H, W, H, W, nullptr, y, nullptr);
+    if (!ok) return cfail(MXP_ECUDA, "launch of a convolution failed");
     net->N = N;
     net->H = H;
     net->W = W;
@@ -259,39 +212,41 @@ mxp_status backward_impl(mxp_cnn *net, const float *x, const float *gy)
 {
     const int N = net->N, H = net->H, W = net->W, H2 = H / 2, W2 = W / 2;
     cudaStream_t st = net->stream;
-    const int64_t full32 = (int64_t)N * 32 * H * W, half64 = (int64_t)N * 64 * H2 * W2;
-    // layer 6
-    conv_bwd_weight<1, 0>(net, 5, net->a[4], N, H, W, gy, H, W);
-    conv_bwd_data<1>(net, 5, gy, N, H, W, H, W, net->g5);            // d/da5
-    // layer 5: a5 = r5 + a1
-    CKC(cudaMemcpyAsync(net->g1, net->g5, full32 * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    count_launch();
-    k_relu_mask<<<ew_grid(full32), 256, 0, st>>>(net->g5, net->r5, full32);
-    conv_bwd_weight<1, 1>(net, 4, net->a[3], N, H2, W2, net->g5, H, W);
-    conv_bwd_data<1>(net, 4, net->g5, N, H, W, H, W, net->gfull);   // d/d up2(a4), full resolution
-    count_launch();
-    k_down2_sum<<<ew_grid(half64), 256, 0, st>>>(net->gfull, N * 64, H2, W2, net->gh);
-    count_launch();
-    k_relu_mask<<<ew_grid(half64), 256, 0, st>>>(net->gh, net->a[3], half64);
+    CKC(cudaMemsetAsync(net->g, 0, net->np * sizeof(float), st));
+    // layer 6; a5 = r5 + a1: its gradient goes on to a1 (g1) and, masked, to layer 5 (g5)
+    bool ok = conv_bwd_weight(net, 5, net->a[4], N, H, W, gy, H, W);
+    ConvOut o;
+    o.out = net->g5;
+    o.out2 = net->g1;
+    o.mask = net->r5;
+    ok = ok && conv_bwd_data(net, 5, gy, N, H, W, H, W, o);
+    // layer 5: the gradient of up2(a4) is summed over 2 x 2 blocks
+    ok = ok && conv_bwd_weight(net, 4, net->a[3], N, H2, W2, net->g5, H, W);
+    o = ConvOut{};
+    o.out = net->gh;
+    o.mask = net->a[3];
+    o.pool = 1;
+    ok = ok && conv_bwd_data(net, 4, net->g5, N, H, W, H, W, o);
     // layer 4
-    conv_bwd_weight<1, 0>(net, 3, net->a[2], N, H2, W2, net->gh, H2, W2);
-    conv_bwd_data<1>(net, 3, net->gh, N, H2, W2, H2, W2, net->gh2);
-    count_launch();
-    k_relu_mask<<<ew_grid(half64), 256, 0, st>>>(net->gh2, net->a[2], half64);
+    ok = ok && conv_bwd_weight(net, 3, net->a[2], N, H2, W2, net->gh, H2, W2);
+    o = ConvOut{};
+    o.out = net->gh2;
+    o.mask = net->a[2];
+    ok = ok && conv_bwd_data(net, 3, net->gh, N, H2, W2, H2, W2, o);
     // layer 3
-    conv_bwd_weight<1, 0>(net, 2, net->a[1], N, H2, W2, net->gh2, H2, W2);
-    conv_bwd_data<1>(net, 2, net->gh2, N, H2, W2, H2, W2, net->gh);
-    count_launch();
-    k_relu_mask<<<ew_grid(half64), 256, 0, st>>>(net->gh, net->a[1], half64);
-    // layer 2 (stride 2)
-    conv_bwd_weight<2, 0>(net, 1, net->a[0], N, H, W, net->gh, H2, W2);
-    conv_bwd_data<2>(net, 1, net->gh, N, H2, W2, H, W, net->g5);
-    count_launch();
-    k_add_to<<<ew_grid(full32), 256, 0, st>>>(net->g5, net->g1, full32);
-    count_launch();
-    k_relu_mask<<<ew_grid(full32), 256, 0, st>>>(net->g5, net->a[0], full32);
+    ok = ok && conv_bwd_weight(net, 2, net->a[1], N, H2, W2, net->gh2, H2, W2);
+    o.out = net->gh;
+    o.mask = net->a[1];
+    ok = ok && conv_bwd_data(net, 2, net->gh2, N, H2, W2, H2, W2, o);
+    // layer 2 (stride 2), plus the skip's gradient
+    ok = ok && conv_bwd_weight(net, 1, net->a[0], N, H, W, net->gh, H2, W2);
+    o.out = net->g5;
+    o.add = net->g1;
+    o.mask = net->a[0];
+    ok = ok && conv_bwd_data(net, 1, net->gh, N, H2, W2, H, W, o);
     // layer 1
-    conv_bwd_weight<1, 0>(net, 0, x, N, H, W, net->g5, H, W);
+    ok = ok && conv_bwd_weight(net, 0, x, N, H, W, net->g5, H, W);
+    if (!ok) return cfail(MXP_ECUDA, "launch of a convolution failed");
     CKC(cudaGetLastError());
     return MXP_OK;
 }
@@ -331,8 +286,7 @@ mxp_status mxp_cnn_create(int device, void *cuda_stream, int max_batch, int max_
     A((void **)&net->a[4], full * 32 * 4); A((void **)&net->r5, full * 32 * 4);
     A((void **)&net->y, full * 2 * 4); A((void **)&net->gy, full * 2 * 4);
     A((void **)&net->g5, full * 32 * 4); A((void **)&net->g1, full * 32 * 4);
-    A((void **)&net->gfull, full * 64 * 4); A((void **)&net->gh, half * 64 * 4);
-    A((void **)&net->gh2, half * 64 * 4);
+    A((void **)&net->gh, half * 64 * 4); A((void **)&net->gh2, half * 64 * 4);
     A((void **)&net->partial, 2048 * sizeof(double)); A((void **)&net->loss_dev, sizeof(float));
     A((void **)&net->err, sizeof(unsigned));
     ok = ok && cudaMallocHost((void **)&net->loss_host, sizeof(float)) == cudaSuccess;
@@ -447,7 +401,7 @@ void mxp_cnn_destroy(mxp_cnn *net)
     if (!net) return;
     cudaStreamSynchronize(net->stream);
     float *bufs[] = {net->w, net->g, net->m, net->v, net->x, net->a[0], net->a[1], net->a[2], net->a[3],
-                     net->a[4], net->r5, net->y, net->gy, net->g5, net->g1, net->gfull, net->gh, net->gh2,
+                     net->a[4], net->r5, net->y, net->gy, net->g5, net->g1, net->gh, net->gh2,
                      net->loss_dev};
     for (float *b : bufs) cudaFree(b);
     cudaFree(net->wb);

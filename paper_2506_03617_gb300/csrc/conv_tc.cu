@@ -1,4 +1,7 @@
-// Tensor-core convolutions of the learned stage (sm_103a, tcgen05).
+// Tensor-core 3x3 convolutions (sm_103a, tcgen05), general form: any number of input
+// channels.  Layers of at most 64 channels on both sides, which is the whole
+// network, run on the tiled kernels of conv_tile.cu (the same results, 4 to 8 times
+// faster); this form has no shared-memory weights and no channel limit.
 //
 // A 3x3 convolution is the contraction D[m][n] = sum_k A[m][k] B[n][k] with
 // m an output pixel, n an output channel and k = (input channel, ky, kx):
@@ -16,7 +19,7 @@
 // the gather of step k + 1 overlaps the MMA of step k.  The epilogue reads the
 // accumulator rows back with tcgen05.ld (warp w owns tensor-memory lanes
 // 32w .. 32w + 31, i.e. pixels 32w .. 32w + 31 of the tile), adds the bias and
-// applies relu / the skip connection.
+// applies relu.
 //
 // Shared-memory operands use the no-swizzle K-major layout: 8 x 16-byte core
 // matrices (8 rows, 8 bfloat16 along K), consecutive along K at LBO = 128 B
@@ -94,7 +97,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 // MODE 0, forward convolution (see cnn.cu for the network):
 //   out[n, co, oy, ox] = act(bias[co] + sum_{ci, ky, kx} W[co, ci, ky, kx] x[n, ci, S oy + ky - 1, S ox + kx - 1])
 //   with x the logical input (nearest-upsampled by 2 when UPS) and zero padding;
-//   out_skip (nullable) = out + skip.  in = x [n][Cin][Hs][Ws], out [n][Cout][Ho][Wo].
+//   in = x [n][Cin][Hs][Ws], out [n][Cout][Ho][Wo].
 // MODE 1, input gradient of that convolution (UPS = 0):
 //   out[n, ci, y, x] = sum_{co, ky, kx} W[co, ci, ky, kx] g[n, co, (y + 1 - ky) / S, (x + 1 - kx) / S]
 //   over the terms whose division is exact and in range.  in = g [n][Cin][Hs][Ws]
@@ -104,9 +107,7 @@ template <int MODE, int S, int UPS, int NT>
 __global__ void __launch_bounds__(128) k_conv_tc(const float *__restrict__ in, int Cin, int Hs, int Ws,
                                                  const __nv_bfloat16 *__restrict__ w,
                                                  const float *__restrict__ bias, int Cout, int Ho, int Wo,
-                                                 int relu, const float *__restrict__ skip,
-                                                 float *__restrict__ out, float *__restrict__ out_skip,
-                                                 int64_t npix, unsigned *err)
+                                                 int relu, float *__restrict__ out, int64_t npix, unsigned *err)
 {
     static_assert(MODE == 0 || (MODE == 1 && UPS == 0), "the input gradient takes no upsampling");
     static_assert(NT == 16 || NT == 32 || NT == 64, "N tile of 16, 32 or 64 channels");
@@ -243,7 +244,6 @@ __global__ void __launch_bounds__(128) k_conv_tc(const float *__restrict__ in, i
                     if (MODE == 0) {
                         if (bias) v += bias[co];
                         if (relu) v = fmaxf(v, 0.f);
-                        if (out_skip) out_skip[q] = v + skip[q];
                     }
                     out[q] = v;
                 }
@@ -389,45 +389,52 @@ __global__ void __launch_bounds__(128) k_conv_wgrad_tc(const float *__restrict__
 
 template <int MODE, int S, int UPS>
 static void launch_tc(int cout, dim3 grid, cudaStream_t st, const float *in, int Cin, int Hs, int Ws,
-                      const __nv_bfloat16 *w, const float *bias, int Ho, int Wo, int relu, const float *skip,
-                      float *out, float *out_skip, int64_t npix, unsigned *err)
+                      const __nv_bfloat16 *w, const float *bias, int Ho, int Wo, int relu, float *out, int64_t npix,
+                      unsigned *err)
 {
     if (cout <= 16)
-        k_conv_tc<MODE, S, UPS, 16><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, skip, out,
-                                                          out_skip, npix, err);
+        k_conv_tc<MODE, S, UPS, 16><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, out, npix, err);
     else if (cout <= 32)
-        k_conv_tc<MODE, S, UPS, 32><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, skip, out,
-                                                          out_skip, npix, err);
+        k_conv_tc<MODE, S, UPS, 32><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, out, npix, err);
     else
-        k_conv_tc<MODE, S, UPS, 64><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, skip, out,
-                                                          out_skip, npix, err);
+        k_conv_tc<MODE, S, UPS, 64><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, out, npix, err);
 }
 
-bool conv_fwd_tc(int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
-                 const float *bias, int Cout, int Ho, int Wo, int relu, const float *skip, float *out,
-                 float *out_skip, unsigned *err, cudaStream_t st)
+static bool conv_fwd_tc(int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
+                        const float *bias, int Cout, int Ho, int Wo, int relu, float *out, unsigned *err,
+                        cudaStream_t st)
 {
-    if (Cout < 1 || Cout > 64 || Cin < 1) return false;
+    if (Cout < 1 || Cout > 64 || Cin < 1 || (UPS && S != 1)) return false;
+    if (conv_tile_fits(Cin, Cout)) {
+        ConvOut o;
+        o.out = out;
+        return conv_tile(false, S, UPS, in, N, Cin, Hs, Ws, w, bias, Cout, Ho, Wo, relu, o, err, st);
+    }
     const int64_t npix = (int64_t)N * Ho * Wo;
     const dim3 grid((unsigned)((npix + 127) / 128));
     count_launch();
-    if (S == 2 && !UPS) launch_tc<0, 2, 0>(Cout, grid, st, in, Cin, Hs, Ws, w, bias, Ho, Wo, relu, skip, out, out_skip, npix, err);
-    else if (S == 1 && UPS) launch_tc<0, 1, 1>(Cout, grid, st, in, Cin, Hs, Ws, w, bias, Ho, Wo, relu, skip, out, out_skip, npix, err);
-    else if (S == 1) launch_tc<0, 1, 0>(Cout, grid, st, in, Cin, Hs, Ws, w, bias, Ho, Wo, relu, skip, out, out_skip, npix, err);
+    if (S == 2 && !UPS) launch_tc<0, 2, 0>(Cout, grid, st, in, Cin, Hs, Ws, w, bias, Ho, Wo, relu, out, npix, err);
+    else if (S == 1 && UPS) launch_tc<0, 1, 1>(Cout, grid, st, in, Cin, Hs, Ws, w, bias, Ho, Wo, relu, out, npix, err);
+    else if (S == 1) launch_tc<0, 1, 0>(Cout, grid, st, in, Cin, Hs, Ws, w, bias, Ho, Wo, relu, out, npix, err);
     else return false;
     return true;
 }
 
-bool conv_bwd_data_tc(int S, const float *gout, int N, int Cout, int Ho, int Wo, const __nv_bfloat16 *w, int Cin,
-                      int Hl, int Wl, float *gin, unsigned *err, cudaStream_t st)
+static bool conv_bwd_data_tc(int S, const float *gout, int N, int Cout, int Ho, int Wo, const __nv_bfloat16 *w,
+                             int Cin, int Hl, int Wl, float *gin, unsigned *err, cudaStream_t st)
 {
     if (Cin < 1 || Cin > 64 || Cout < 1) return false;
+    if (conv_tile_fits(Cout, Cin)) {
+        ConvOut o;
+        o.out = gin;
+        return conv_tile(true, S, 0, gout, N, Cout, Ho, Wo, w, nullptr, Cin, Hl, Wl, 0, o, err, st);
+    }
     const int64_t npix = (int64_t)N * Hl * Wl;
     const dim3 grid((unsigned)((npix + 127) / 128));
     count_launch();
     // the GEMM's K side is the layer's output channels, its N side the input channels
-    if (S == 2) launch_tc<1, 2, 0>(Cin, grid, st, gout, Cout, Ho, Wo, w, nullptr, Hl, Wl, 0, nullptr, gin, nullptr, npix, err);
-    else if (S == 1) launch_tc<1, 1, 0>(Cin, grid, st, gout, Cout, Ho, Wo, w, nullptr, Hl, Wl, 0, nullptr, gin, nullptr, npix, err);
+    if (S == 2) launch_tc<1, 2, 0>(Cin, grid, st, gout, Cout, Ho, Wo, w, nullptr, Hl, Wl, 0, gin, npix, err);
+    else if (S == 1) launch_tc<1, 1, 0>(Cin, grid, st, gout, Cout, Ho, Wo, w, nullptr, Hl, Wl, 0, gin, npix, err);
     else return false;
     return true;
 }
@@ -449,14 +456,16 @@ static void launch_wgrad(int cout, dim3 grid, cudaStream_t st, const float *x, i
         k_conv_wgrad_tc<S, UPS, 64, kWgradSteps><<<grid, 128, 0, st>>>(x, Cin, Hs, Ws, g, cout, Ho, Wo, npix, gw, err);
 }
 
-bool conv_wgrad_tc(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
-                   int Wo, float *gw, unsigned *err, cudaStream_t st)
+static bool conv_wgrad_tc(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout,
+                          int Ho, int Wo, float *gw, unsigned *err, cudaStream_t st)
 {
     if (Cout < 1 || Cout > 64 || Cin < 1) return false;
     const int64_t npix = (int64_t)N * Ho * Wo;
     const int K = Cin * 9;
     const dim3 grid((unsigned)((npix + kWgradSteps * 16 - 1) / (kWgradSteps * 16)), (unsigned)((K + 127) / 128));
     if (cudaMemsetAsync(gw, 0, (size_t)Cout * K * sizeof(float), st) != cudaSuccess) return false;
+    if (conv_tile_fits(Cin, Cout))
+        return wgrad_tile(S, UPS, x, N, Cin, Hs, Ws, g, Cout, Ho, Wo, gw, nullptr, err, st);
     count_launch();
     if (S == 2 && !UPS) launch_wgrad<2, 0>(Cout, grid, st, x, Cin, Hs, Ws, g, Ho, Wo, npix, gw, err);
     else if (S == 1 && UPS) launch_wgrad<1, 1>(Cout, grid, st, x, Cin, Hs, Ws, g, Ho, Wo, npix, gw, err);
@@ -500,8 +509,7 @@ extern "C" mxp_status mxp_cnn_conv3x3(int mode, int stride, int upsample, int N,
     const __nv_bfloat16 *w = static_cast<const __nv_bfloat16 *>(w_bf16_dev);
     bool ok = false;
     if (mode == 0)
-        ok = conv_fwd_tc(stride, upsample, a_dev, N, Cin, Hs, Ws, w, bias_dev, Cout, Ho, Wo, relu, nullptr, out_dev,
-                         nullptr, err, st);
+        ok = conv_fwd_tc(stride, upsample, a_dev, N, Cin, Hs, Ws, w, bias_dev, Cout, Ho, Wo, relu, out_dev, err, st);
     else if (mode == 1)
         ok = conv_bwd_data_tc(stride, a_dev, N, Cout, Ho, Wo, w, Cin, Hs, Ws, out_dev, err, st);
     else

@@ -293,25 +293,26 @@ void hess_start(const HessState &hs, cudaStream_t st);
 // Solve the j x j upper-triangular system H y = g into hs.y.
 void hess_backsolve(const HessState &hs, int j, cudaStream_t st);
 
-// Tensor-core (tcgen05) forward 3x3 convolution of the learned stage (conv_tc.cu):
-// stride S (1 or 2), input nearest-upsampled by 2 when UPS, Cout <= 64;
-// *err receives 1 when a bounded wait gives up.  Returns false for an
-// unsupported shape.
-bool conv_fwd_tc(int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
-                 const float *bias, int Cout, int Ho, int Wo, int relu, const float *skip, float *out,
-                 float *out_skip, unsigned *err, cudaStream_t st);
-
-// Tensor-core input gradient of a 3x3 convolution of stride S (conv_tc.cu):
-// gin [N][Cin][Hl][Wl] from gout [N][Cout][Ho][Wo] and the layer's weights
-// W [Cout][Cin][3][3]; Cin <= 64.
-bool conv_bwd_data_tc(int S, const float *gout, int N, int Cout, int Ho, int Wo, const __nv_bfloat16 *w, int Cin,
-                      int Hl, int Wl, float *gin, unsigned *err, cudaStream_t st);
-
-// Tensor-core weight gradient of a 3x3 convolution (conv_tc.cu): gw [Cout][Cin * 9]
-// = sum over pixels of im2col(x) x g (x the layer input [N][Cin][Hs][Ws], upsampled
-// when UPS; g the output gradient [N][Cout][Ho][Wo]); Cout <= 64.  Overwrites gw.
-bool conv_wgrad_tc(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
-                   int Wo, float *gw, unsigned *err, cudaStream_t st);
+// Tensor-core (tcgen05) 3x3 convolutions of at most 64 channels on both sides
+// (conv_tile.cu), stride S (1 or 2), forward with the input nearest-upsampled by 2
+// when UPS; *err receives 1 when a bounded wait gives up.  Where the result goes:
+//   forward: out = act(bias + conv), out2 (nullable) = out + add
+//   input gradient: v = gradient + add (nullable); out2 (nullable) = v; out = v where
+//   mask (nullable) > 0, else 0.  pool: v is first summed over 2 x 2 blocks (even Ho,
+//   Wo; the adjoint of nearest upsampling); no add or out2.
+struct ConvOut {
+    float *out = nullptr, *out2 = nullptr;
+    const float *add = nullptr, *mask = nullptr;
+    int pool = 0;
+};
+bool conv_tile_fits(int Cin, int Cout);
+// grad = false: in [N][Cin][Hs][Ws] -> [N][Cout][Ho][Wo], weights W [Cout][Cin][3][3];
+// grad = true: in the output gradient, weights W [Cin][Cout][3][3].
+bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
+               const float *bias, int Cout, int Ho, int Wo, int relu, const ConvOut &o, unsigned *err, cudaStream_t st);
+// Adds the weight gradient to gw (and the sums of g per channel to gb, nullable).
+bool wgrad_tile(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
+                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st);
 
 // Learned stage: z = network(v) on a 2D grid (n0 x n1), see cnn.cu.
 mxp_status cnn_apply_vector(mxp_cnn *net, int n0, int n1, const double2 *v, double vnorm,
