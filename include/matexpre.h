@@ -330,6 +330,9 @@ typedef enum {
     MXP_SWEEP_ZMARCH_3D = 4,      /* one launch per step, threads march along z in registers */
     MXP_SWEEP_ZMARCH_TMA_3D = 5   /* one launch per step, planes staged by TMA (n0 % 4 == 0) */
 } mxp_sweep_kind;
+/* With fuse_k = 0 the exp actions of the two z-marching kinds take two steps per
+ * launch (planes staged by TMA, rows padded where n0 % 4 != 0); the results are those
+ * of single steps to the last bit. */
 /* Returns an mxp_sweep_kind, or -1 for a NULL problem or a failed set-up.
  * For 3D low-precision problems it may allocate the problem's work buffers and
  * build their TMA descriptors (as the first action would). */

@@ -108,9 +108,11 @@ struct mxp_problem {
     float2 *face32 = nullptr;
     float2 *face32s = nullptr;            // face32 scaled by h^2 (persistent kernel)
     int64_t face_off[6] = {0, 0, 0, 0, 0, 0};
-    // tensor maps of the TMA-staged 3D sweep (built on first use per precision)
+    // tensor maps of the TMA-staged 3D sweeps (built on first use per precision)
     Tma3Maps *tma3 = nullptr;
     int tma3_prec = -1;                  // precision the maps (or their absence) belong to
+    float *kappa_pad = nullptr;          // kappa32 with padded rows, when n0 is no multiple of 4
+    bool kappa_pad_ok = false;
     std::vector<double2> coef_host;   // [3][3][nmax]
     // shift and plans
     double mu = 0;
@@ -328,6 +330,7 @@ static mxp_status upload_coefs(mxp_problem *P)
     for (size_t i = 0; i < cnt; ++i) c64[i] = make_double2(P->coef_host[i].x * h2, P->coef_host[i].y * h2);
     CK(cudaMemcpyAsync(P->coef64, c64.data(), cnt * sizeof(double2), cudaMemcpyHostToDevice, P->stream));
     compute_kappa(P->c_dev, P->prm.omega, P->kappa64, P->kappa32, P->ntot, P->stream);
+    P->kappa_pad_ok = false;
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(P->stream));
     return MXP_OK;
@@ -821,17 +824,36 @@ static mxp_status retune(mxp_problem *P)
     return MXP_OK;
 }
 
-// which = 0: out = exp(i t A_s) x; which = 1: out = psi_1(i t A_s) x.
-// out_mode 1 returns x - result instead (the fixed-point operator of Eq. fixed-point).
-// Tensor maps for the TMA-staged 3D sweep of this problem, or nullptr when the
+// Whether the 3D exp actions take two steps per launch (tma3d2.cu): unless the
+// parameters ask for unfused sweeps (fuse_k = 1).
+static bool tma3_two(const mxp_problem *P) { return P->prm.fuse_k == 0; }
+
+// Tensor maps for the TMA-staged 3D sweeps of this problem, or nullptr when the
 // grid or the driver does not allow them (the register-marching sweep is used).
+// Rows that are no multiple of 4 are padded for the two-step sweeps; single-step
+// sweeps and psi actions of such grids march in registers.
 template <typename S>
-static const Tma3Maps *tma3_maps(mxp_problem *P)
+static const Tma3Maps *tma3_maps(mxp_problem *P, bool padded)
 {
     if (P->grid.dim != 3 || P->nfaces) return nullptr;
+    const int n0 = P->geom.n[0], pitch = tma3_pitch(P->geom);
+    if (pitch != n0 && !padded) return nullptr;
+    const int64_t rows = (int64_t)P->geom.n[1] * P->geom.n[2];
+    if (pitch > n0 && !P->kappa_pad_ok) {
+        if (!P->kappa_pad && cudaMalloc(&P->kappa_pad, (size_t)rows * pitch * sizeof(float)) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (cudaMemcpy2DAsync(P->kappa_pad, pitch * sizeof(float), P->kappa32, n0 * sizeof(float), n0 * sizeof(float),
+                              (size_t)rows, cudaMemcpyDeviceToDevice, P->stream) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        P->kappa_pad_ok = true;
+    }
     if (P->tma3_prec == (int)P->prm.prec) return P->tma3;
     tma3_destroy(P->tma3);
-    P->tma3 = tma3_create<S>(P->geom, P->hb, P->kappa32);
+    P->tma3 = tma3_create<S>(P->geom, P->hb, pitch > n0 ? P->kappa_pad : P->kappa32);
     P->tma3_prec = (int)P->prm.prec;
     return P->tma3;
 }
@@ -865,6 +887,8 @@ struct AugScalars {
     void end_substep() { z1 = g1; z2 = g2; }
 };
 
+// which = 0: out = exp(i t A_s) x; which = 1: out = psi_1(i t A_s) x.
+// out_mode 1 returns x - result instead (the fixed-point operator of Eq. fixed-point).
 template <typename S>
 static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *out, int out_mode)
 {
@@ -874,12 +898,20 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
     S *vs = (S *)P->hb[3];
     const int64_t n = P->ntot;
     cudaStream_t st = P->stream;
-    if (which == 0) {
-        launch_convert_in<S>(x, b[0], n, st);
-    } else {
-        launch_convert_in<S>(x, vs, n, st);
-        cudaMemsetAsync(b[0], 0, (size_t)n * sizeof(S), st);
+    // 3D complex64 / bf16: planes staged by TMA (b[i] is work buffer i, v is buffer 3),
+    // rows padded where n0 is no multiple of 4
+    const Tma3Maps *tm = nullptr;
+    if constexpr (sizeof(S) <= 8) {
+        if (P->grid.dim == 3 && !(which == 0 && P->f3_cfg >= 0 && pl.m % fused3d_cfg_k(P->f3_cfg) == 0))
+            tm = tma3_maps<S>(P, which == 0 && tma3_two(P));
     }
+    const int n0 = P->geom.n[0], pitch = tm ? tma3_maps_pitch(tm) : n0;
+    const int64_t nrow = n / n0;
+    if constexpr (sizeof(S) <= 8) {
+        if (pitch != n0) launch_convert_in_rows<S>(x, which ? vs : b[0], n0, nrow, pitch, st);
+    }
+    if (pitch == n0) launch_convert_in<S>(x, which ? vs : b[0], n, st);
+    if (which) cudaMemsetAsync(b[0], 0, (size_t)nrow * pitch * sizeof(S), st);
     const double t = P->prm.t;
     const int Ssub = pl.S, m = pl.m;
     const cd rot(0.0, -t * P->mu / Ssub);                 // scalar row of the augmented matrix / S
@@ -996,36 +1028,50 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
         P->passes += passes;
         return passes;
     }
+    const bool two = tm && which == 0 && tma3_two(P);
     for (int sub = 0; sub < Ssub; ++sub) {
         int in = iy;
         aug.begin_substep();
-        for (int k = m; k >= 1; --k) {
-            sc.sigma = PrecData<S>::c(cd(0.0, t / ((double)Ssub * k)));
-            sc.gamma = PrecData<S>::c(aug.gamma(k));
-            sc.rho = PrecData<S>::c((sub == Ssub - 1 && k == 1) ? final_rho : cd(1.0));
+        for (int k = m; k >= 1;) {
+            const int steps = two && k >= 2 ? 2 : 1;
+            StepScalars<C> s1 = sc;              // first of two steps
+            for (int s = 0; s < steps; ++s, --k) {
+                sc.sigma = PrecData<S>::c(cd(0.0, t / ((double)Ssub * k)));
+                sc.gamma = PrecData<S>::c(aug.gamma(k));
+                sc.rho = PrecData<S>::c((sub == Ssub - 1 && k == 1) ? final_rho : cd(1.0));
+                aug.step(k);
+                if (s == 0) s1 = sc;
+            }
             const int o = (in == iy) ? (iy + 1) % 3 : 3 - iy - in;
-            bool done = false;
             if constexpr (sizeof(S) <= 8) {
-                // 3D complex64 / bf16: planes staged by TMA (b[i] is work buffer i, v is buffer 3)
-                if (const Tma3Maps *tm = tma3_maps<S>(P)) {
-                    const cudaError_t ce = launch_step3z_tma<S>(P->geom, PrecData<S>::coef(P), sc, tm, in, iy,
-                                                                which ? 3 : -1, b[o], P->bar + 2, st);
-                    if (ce != cudaSuccess) {
-                        fail(MXP_ECUDA, std::string("TMA 3D sweep: ") + cudaGetErrorString(ce));
-                        return -1;
-                    }
-                    done = true;
+                cudaError_t ce = cudaSuccess;
+                if (steps == 2) {
+                    ce = launch_step3z2<S>(P->geom, PrecData<S>::coef(P), s1, sc, tm, in, iy, b[o], P->bar + 2, st, passes > 0);
+                } else if (tm && pitch == n0) {
+                    ce = launch_step3z_tma<S>(P->geom, PrecData<S>::coef(P), sc, tm, in, iy, which ? 3 : -1, b[o], P->bar + 2,
+                                              st);
+                } else if (tm) {                 // the last step of an odd degree on padded rows
+                    Geom gp = P->geom;
+                    gp.s1 = pitch;
+                    gp.s2 = (int64_t)pitch * gp.n[1];
+                    launch_step<S>(gp, PrecData<S>::coef(P), P->kappa_pad, sc, b[in], b[iy], nullptr, b[o], st);
+                }
+                if (ce != cudaSuccess) {
+                    fail(MXP_ECUDA, std::string("TMA 3D sweep: ") + cudaGetErrorString(ce));
+                    return -1;
                 }
             }
-            if (!done) sweep<S>(P, sc, b[in], b[iy], which ? vs : nullptr, b[o], st, passes > 0);
-            aug.step(k);
+            if (!tm) sweep<S>(P, sc, b[in], b[iy], which ? vs : nullptr, b[o], st, passes > 0);
             in = o;
-            ++passes;
+            passes += steps;
         }
         iy = in;
         aug.end_substep();
     }
-    launch_convert_out<S>(b[iy], out, x, out_mode, n, st);
+    if constexpr (sizeof(S) <= 8) {
+        if (pitch != n0) launch_convert_out_rows<S>(b[iy], out, x, out_mode, n0, nrow, pitch, st);
+    }
+    if (pitch == n0) launch_convert_out<S>(b[iy], out, x, out_mode, n, st);
     P->passes += passes;
     return passes;
 }
@@ -2448,7 +2494,7 @@ int mxp_sweep_kernel(mxp_problem *P)
     if (P->nfaces) return MXP_SWEEP_POINTWISE;
     DeviceGuard guard(P->device);
     if (ensure_base(P) != MXP_OK) return -1;
-    const Tma3Maps *tm = (P->prm.prec == MXP_C64) ? tma3_maps<float2>(P) : tma3_maps<__nv_bfloat162>(P);
+    const Tma3Maps *tm = (P->prm.prec == MXP_C64) ? tma3_maps<float2>(P, false) : tma3_maps<__nv_bfloat162>(P, false);
     return tm ? MXP_SWEEP_ZMARCH_TMA_3D : MXP_SWEEP_ZMARCH_3D;
 }
 
@@ -2768,6 +2814,7 @@ void mxp_destroy(mxp_problem *P)
     cudaFree(P->face64); cudaFree(P->face32); cudaFree(P->face32s);
     for (int i = 0; i < 4; ++i) cudaFree(P->hb[i]);
     tma3_destroy(P->tma3);
+    cudaFree(P->kappa_pad);
     cudaFree(P->rt); cudaFree(P->tmp); cudaFree(P->tmp2); cudaFree(P->bdev); cudaFree(P->xdev);
     cudaFree(P->ks.partials);
     cudaFree(P->vec_dev);

@@ -115,14 +115,22 @@ template <typename C> struct StepScalars {
     int nfaces = 0;
 };
 
-// TMA-staged 3D sweep (tma3d.cu): tensor maps of the four 16-byte-per-unknown
-// work buffers (as p with halo and as y / v tiles) and of kappa; nullptr when
-// the grid does not qualify (3D with n0 a multiple of 4, 16-byte aligned
-// buffers) or the driver offers no tensor-map encoder.
+// TMA-staged 3D sweeps (tma3d.cu, tma3d2.cu): tensor maps of the four
+// 16-byte-per-unknown work buffers and of kappa, all with rows of tma3_pitch(g)
+// values; nullptr when the grid does not qualify (pitch 0), a buffer is not 16-byte
+// aligned, or the driver offers no tensor-map encoder.
 struct Tma3Maps;
+int tma3_pitch(const Geom &g);
+int tma3_maps_pitch(const Tma3Maps *t);
 template <typename S>
 Tma3Maps *tma3_create(const Geom &g, void *const *bufs, const float *kappa);
 void tma3_destroy(Tma3Maps *t);
+// Two consecutive steps of one sub-step without a psi source (s1, then s2; only s2's rho
+// counts): q = step of p with y, out = step of q with y.  chain: the launch may start before the kernel
+// launched before it on st has ended.
+template <typename S>
+cudaError_t launch_step3z2(const Geom &g, const float2 *coef, const StepScalars<float2> &s1, const StepScalars<float2> &s2,
+                           const Tma3Maps *t, int ip, int iy, S *pout, unsigned *err, cudaStream_t st, bool chain);
 // pout = one Taylor-Horner step as launch_step, reading p from buffer ip, y
 // from buffer iy and v from buffer iv (-1 = none); err receives 1 on a wait
 // timeout.
@@ -236,6 +244,12 @@ cudaError_t barrier_selftest(unsigned *bar, cudaStream_t st);
 
 template <typename S>
 void launch_convert_in(const double2 *x, S *out, int64_t n, cudaStream_t st);
+// the same for `rows` rows of n0 values, the stored side's rows `pitch` values apart
+template <typename S>
+void launch_convert_in_rows(const double2 *x, S *out, int n0, int64_t rows, int pitch, cudaStream_t st);
+template <typename S>
+void launch_convert_out_rows(const S *x, double2 *out, const double2 *base, int mode, int n0, int64_t rows, int pitch,
+                             cudaStream_t st);
 // out = x (mode 0) or out = base - x (mode 1), both complex128
 template <typename S>
 void launch_convert_out(const S *x, double2 *out, const double2 *base, int mode, int64_t n,

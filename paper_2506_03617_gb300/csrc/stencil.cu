@@ -243,6 +243,27 @@ __global__ void k_convert_out(const S *__restrict__ x, double2 *__restrict__ out
     }
 }
 
+// Rows of n0 values on one side, of `pitch` on the stored side: a warp per row.
+template <typename S>
+__global__ void k_convert_in_rows(const double2 *__restrict__ x, S *__restrict__ out, int n0, int64_t rows, int pitch)
+{
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.y + threadIdx.y; r < rows; r += (int64_t)gridDim.x * blockDim.y)
+        for (int i = threadIdx.x; i < n0; i += 32) St<S>::st(out, r * pitch + i, St<S>::from64(x[r * n0 + i]));
+}
+
+template <typename S>
+__global__ void k_convert_out_rows(const S *__restrict__ x, double2 *__restrict__ out, const double2 *__restrict__ base,
+                                   int mode, int n0, int64_t rows, int pitch)
+{
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.y + threadIdx.y; r < rows; r += (int64_t)gridDim.x * blockDim.y)
+        for (int i = threadIdx.x; i < n0; i += 32) {
+            const auto c = St<S>::ld(x, r * pitch + i);
+            double2 v = make_double2((double)c.x, (double)c.y);
+            if (mode == 1) v = csub(base[r * n0 + i], v);
+            out[r * n0 + i] = v;
+        }
+}
+
 static int stream_grid(int64_t n)
 {
     int64_t b = (n + 255) / 256;
@@ -266,10 +287,28 @@ void launch_convert_out(const S *x, double2 *out, const double2 *base, int mode,
     k_convert_out<S><<<stream_grid(n), 256, 0, st>>>(x, out, base, mode, n);
 }
 
+template <typename S>
+void launch_convert_in_rows(const double2 *x, S *out, int n0, int64_t rows, int pitch, cudaStream_t st)
+{
+    count_launch();
+    k_convert_in_rows<S><<<stream_grid(rows * 32), dim3(32, 8), 0, st>>>(x, out, n0, rows, pitch);
+}
+
+template <typename S>
+void launch_convert_out_rows(const S *x, double2 *out, const double2 *base, int mode, int n0, int64_t rows, int pitch,
+                             cudaStream_t st)
+{
+    count_launch();
+    k_convert_out_rows<S><<<stream_grid(rows * 32), dim3(32, 8), 0, st>>>(x, out, base, mode, n0, rows, pitch);
+}
+
 #define MXP_INST_STEP(S)                                                                     \
     template void launch_step<S>(const Geom &, const St<S>::C *, const St<S>::R *,           \
                                  const StepScalars<St<S>::C> &, const S *, const S *,        \
-                                 const S *, S *, cudaStream_t);
+                                 const S *, S *, cudaStream_t);                              \
+    template void launch_convert_in_rows<S>(const double2 *, S *, int, int64_t, int, cudaStream_t); \
+    template void launch_convert_out_rows<S>(const S *, double2 *, const double2 *, int, int, int64_t, int, \
+                                             cudaStream_t);
 #define MXP_INST(S)                                                                          \
     template void launch_convert_in<S>(const double2 *, S *, int64_t, cudaStream_t);         \
     template void launch_convert_out<S>(const S *, double2 *, const double2 *, int, int64_t, \

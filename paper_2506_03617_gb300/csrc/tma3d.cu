@@ -17,8 +17,8 @@
 // are viewed as arrays of 4-byte elements (a complex64 value is two of them, a
 // bf16x2 value one), the tile starts at x0 (a multiple of 32) and its left halo
 // is widened to 2 (complex64) or 4 (bf16x2) cells, so every x start is a
-// multiple of 16 bytes.  Row strides must be multiples of 16 bytes, which holds
-// when n0 is a multiple of 4; other grids use the register-marching sweep.
+// multiple of 16 bytes.  Row strides must be multiples of 16 bytes: the buffers' rows
+// are n0 rounded up to a multiple of 4 values apart.
 //
 // Every wait on an mbarrier is bounded: on timeout the kernel sets the error
 // word (reported as MXP_ETIMEOUT), stops issuing loads, waits (again bounded) for
@@ -29,6 +29,7 @@
 #include <mutex>
 
 #include "mxp_internal.h"
+#include "tma3.h"
 
 #ifndef MXP_TMA3_STAGES
 #define MXP_TMA3_STAGES 6
@@ -42,15 +43,6 @@ namespace mxp {
 constexpr int kRPT = MXP_TMA3_RPT;        // rows of the tile per thread
 constexpr int kTX = 32, kTY = 8 * kRPT;   // tile of a block (32 x 8 threads)
 constexpr int kStages = MXP_TMA3_STAGES;  // planes resident or in flight per block
-constexpr long long kTmaPollLimit = 1ll << 22;
-
-template <typename S> struct TmaElt;
-template <> struct TmaElt<float2> {        // complex64: two 4-byte elements per value
-    static constexpr int E = 2, HL = 2;
-};
-template <> struct TmaElt<__nv_bfloat162> {  // bf16x2: one 4-byte element per value
-    static constexpr int E = 1, HL = 4;
-};
 
 template <typename S> struct Tma3Geo {
     static constexpr int PW = kTX + 2 * TmaElt<S>::HL;   // p tile row, in values
@@ -67,44 +59,6 @@ template <typename S> struct Tma3Geo {
         return PBYTES + (has_y ? YBYTES : 0) + KBYTES + (has_v ? YBYTES : 0);
     }
 };
-
-__device__ __forceinline__ unsigned smem_u32(const void *p)
-{
-    return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void tma_load3(void *dst, const CUtensorMap *map, int c0, int c1, int c2,
-                                          unsigned long long *bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];"
-        :
-        : "r"(smem_u32(dst)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(c0), "r"(c1), "r"(c2),
-          "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect(unsigned long long *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// true once the phase with the given parity has completed; false after the limit
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity)
-{
-    for (long long it = 0; it < kTmaPollLimit; ++it) {
-        unsigned done;
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(done)
-            : "r"(smem_u32(bar)), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 
 template <typename C>
 __device__ __forceinline__ C czero3() { return CT<C>::mk(0, 0); }
@@ -192,7 +146,7 @@ __global__ void __launch_bounds__(kTX * 8) k_step3z_tma(Geom g, const typename S
         xyin[rr] = g.fast && i >= p0 && i < n0 - p0 && j >= p0 && j < n1 - p0;
     }
     int sm_ = 0, sc_ = 1, sp_ = 2;            // stages of planes pi - 1, pi, pi + 1
-    S *outp = pout + (i + g.s1 * (y0 + ty) + g.s2 * z0);
+    S *outp = pout + (i + g.s1 * (y0 + ty) + g.s2 * z0);   // g's strides: the padded rows'
     // z-axis coefficients of the current plane, loaded one plane ahead
     C czp = cz[z0], czm = cz[nm + z0], czc = cz[2 * nm + z0];
 
@@ -292,13 +246,13 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-// 3D map of a grid-shaped array of 4-byte elements (e per value), box bx x by x 1
-static bool encode3(CUtensorMap *m, const void *base, const Geom &g, int e, int bx, int by)
+bool tma3_encode(CUtensorMap *m, const void *base, int64_t ex, int64_t ey, int64_t ez, int64_t row, int64_t plane, int bx,
+                 int by)
 {
     auto fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)g.n[0] * e, (cuuint64_t)g.n[1], (cuuint64_t)g.n[2]};
-    const cuuint64_t strides[2] = {(cuuint64_t)g.n[0] * e * 4, (cuuint64_t)g.n[0] * g.n[1] * e * 4};
+    const cuuint64_t dims[3] = {(cuuint64_t)ex, (cuuint64_t)ey, (cuuint64_t)ez};
+    const cuuint64_t strides[2] = {(cuuint64_t)row, (cuuint64_t)plane};
     const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
     const cuuint32_t es[3] = {1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims, strides, box, es,
@@ -306,26 +260,31 @@ static bool encode3(CUtensorMap *m, const void *base, const Geom &g, int e, int 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-struct Tma3Maps {
-    CUtensorMap p[4], y[4], k;
-    bool ok = false;
-};
+int tma3_pitch(const Geom &g)
+{
+    const int pitch = (g.n[0] + 3) / 4 * 4;
+    // the work buffers hold 16 bytes an unknown, a low-precision value at most 8
+    return g.dim == 3 && pitch <= 2 * g.n[0] ? pitch : 0;
+}
 
 template <typename S>
 Tma3Maps *tma3_create(const Geom &g, void *const *bufs, const float *kappa)
 {
-    if (g.dim != 3 || g.n[0] % 4 != 0) return nullptr;
-    if ((reinterpret_cast<uintptr_t>(kappa) & 15) != 0) return nullptr;
+    const int pitch = tma3_pitch(g);
+    if (!pitch || (reinterpret_cast<uintptr_t>(kappa) & 15) != 0) return nullptr;
     for (int b = 0; b < 4; ++b)
         if ((reinterpret_cast<uintptr_t>(bufs[b]) & 15) != 0) return nullptr;
     constexpr int E = TmaElt<S>::E, HL = TmaElt<S>::HL;
     Tma3Maps *t = new Tma3Maps();
+    t->pitch = pitch;
+    const int64_t row = (int64_t)pitch * E * 4, plane = row * g.n[1], krow = (int64_t)pitch * 4, kplane = krow * g.n[1];
     bool ok = true;
     for (int b = 0; b < 4 && ok; ++b) {
-        ok = encode3(&t->p[b], bufs[b], g, E, E * (kTX + 2 * HL), kTY + 2) &&
-             encode3(&t->y[b], bufs[b], g, E, E * kTX, kTY);
+        ok = tma3_encode(&t->p[b], bufs[b], (int64_t)g.n[0] * E, g.n[1], g.n[2], row, plane, E * (kTX + 2 * HL), kTY + 2) &&
+             tma3_encode(&t->y[b], bufs[b], (int64_t)g.n[0] * E, g.n[1], g.n[2], row, plane, E * kTX, kTY);
     }
-    ok = ok && encode3(&t->k, kappa, g, 1, kTX, kTY);
+    ok = ok && tma3_encode(&t->k, kappa, g.n[0], g.n[1], g.n[2], krow, kplane, kTX, kTY) &&
+         tma3_maps2<S>(t, g, bufs, kappa);
     if (!ok) {
         delete t;
         return nullptr;
@@ -335,6 +294,8 @@ Tma3Maps *tma3_create(const Geom &g, void *const *bufs, const float *kappa)
 }
 
 void tma3_destroy(Tma3Maps *t) { delete t; }
+
+int tma3_maps_pitch(const Tma3Maps *t) { return t ? t->pitch : 0; }
 
 template <typename S, bool HAS_Y, bool HAS_V>
 static cudaError_t launch3t(const Geom &g, const typename St<S>::C *coef, const StepScalars<typename St<S>::C> &sc,
@@ -367,10 +328,13 @@ cudaError_t launch_step3z_tma(const Geom &g, const typename St<S>::C *coef, cons
                               const Tma3Maps *t, int ip, int iy, int iv, S *pout, unsigned *err, cudaStream_t st)
 {
     if (!t || !t->ok || ip < 0 || ip > 3 || iy > 3 || iv > 3) return cudaErrorInvalidValue;
-    if (iy >= 0 && iv >= 0) return launch3t<S, true, true>(g, coef, sc, *t, ip, iy, iv, pout, err, st);
-    if (iy >= 0) return launch3t<S, true, false>(g, coef, sc, *t, ip, iy, iv, pout, err, st);
-    if (iv >= 0) return launch3t<S, false, true>(g, coef, sc, *t, ip, 0, iv, pout, err, st);
-    return launch3t<S, false, false>(g, coef, sc, *t, ip, 0, iv, pout, err, st);
+    Geom gp = g;
+    gp.s1 = t->pitch;
+    gp.s2 = (int64_t)t->pitch * g.n[1];
+    if (iy >= 0 && iv >= 0) return launch3t<S, true, true>(gp, coef, sc, *t, ip, iy, iv, pout, err, st);
+    if (iy >= 0) return launch3t<S, true, false>(gp, coef, sc, *t, ip, iy, iv, pout, err, st);
+    if (iv >= 0) return launch3t<S, false, true>(gp, coef, sc, *t, ip, 0, iv, pout, err, st);
+    return launch3t<S, false, false>(gp, coef, sc, *t, ip, 0, iv, pout, err, st);
 }
 
 #define MXP_TINST(S)                                                                                     \
