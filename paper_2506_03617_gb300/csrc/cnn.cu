@@ -162,7 +162,7 @@ bool conv_fwd(const mxp_cnn *net, int l, const float *in, int N, int Hs, int Ws,
     o.out2 = out2;
     o.add = skip;
     return conv_tile(false, L.stride, L.ups, in, N, L.cin, Hs, Ws, w, net->w + layer_woff(l) + (int64_t)L.cin * L.cout * 9,
-                     L.cout, Ho, Wo, L.relu, o, net->err, net->stream);
+                     L.cout, Ho, Wo, L.relu, o, net->err, net->stream, l > 0);
 }
 
 // gradient of layer l's (logical) input, to o
@@ -170,7 +170,7 @@ bool conv_bwd_data(const mxp_cnn *net, int l, const float *gout, int N, int Ho, 
 {
     const CnnLayer L = kNet[l];
     return conv_tile(true, L.stride, 0, gout, N, L.cout, Ho, Wo, net->wb + layer_woff(l), nullptr, L.cin, Hl, Wl, 0, o,
-                     net->err, net->stream);
+                     net->err, net->stream, true);
 }
 
 // adds layer l's weight and bias gradients to net->g
@@ -180,7 +180,7 @@ bool conv_bwd_weight(const mxp_cnn *net, int l, const float *xin, int N, int Hs,
     const CnnLayer L = kNet[l];
     float *gw = net->g + layer_woff(l);
     return wgrad_tile(L.stride, L.ups, xin, N, L.cin, Hs, Ws, gout, L.cout, Ho, Wo, gw,
-                      gw + (int64_t)L.cin * L.cout * 9, net->err, net->stream);
+                      gw + (int64_t)L.cin * L.cout * 9, net->err, net->stream, l < 5);
 }
 
 mxp_status check_shape(const mxp_cnn *net, int N, int H, int W)

@@ -32,9 +32,10 @@
 // 211 us, 206 TFLOP/s): the issue of the MMAs, 62 cycles each
 // whatever N is (135 us), under the stores of A (150 us without the loads); the loads'
 // latency adds 40 us, the epilogue 8 us.  The weights and the launch cost 12 us a
-// kernel, which is most of a layer on a batch of 32 crops of 64 x 64.  One forward pass
-// on 1088^2: 0.72 ms, before 2.98 ms; forward and gradients of the batch: 0.57 ms,
-// before 4.27 ms.
+// kernel, which is most of a layer on a batch of 32 crops of 64 x 64; as dependent
+// launches they run under the kernel before (0.57 -> 0.52 ms for forward and gradients
+// of that batch, before these kernels 4.28 ms).  One forward pass on 1088^2: 0.70 ms,
+// before 2.98 ms.
 //
 // Every wait on an mbarrier is bounded; on timeout the kernel sets *err, all roles
 // leave their loops, the issuer waits (bounded) for its last commit, and the
@@ -106,6 +107,11 @@ __device__ __forceinline__ bool all_of_128(bool ok)
         : "memory");
     return r != 0;
 }
+
+// Programmatic dependent launch: the next kernel's set-up (barriers, tensor memory,
+// weights) may run under this kernel's last tiles; its activations wait for this one.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -259,6 +265,7 @@ struct ConvArgs {
     ConvOut o;
     int ntx, nty, ntiles;
     int NT, KT;              // N tile (16, 32, 64); k rows in all, padded per stage
+    bool chain;
     unsigned *err;
 };
 
@@ -500,6 +507,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
         for (int i = tid; i < kSlots * 2 * kBlk / 16; i += kThreads) reinterpret_cast<uint4 *>(sA)[i] = make_uint4(0, 0, 0, 0);
         fence_async_smem();
     }
+    let_next_start();
     tc_before();
     __syncthreads();
     tc_after();
@@ -546,6 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
             at.next(nst);
             return true;
         };
+        wait_for_previous();
 #pragma unroll
         for (int d = 0; d < D; ++d) load(q[d]);
         // buffers by name, not shifted: a move of a value still in flight would wait for it
@@ -605,6 +614,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
         __syncwarp();
         if (lane == 0) bar_arrive(&sh.wready);
         asm volatile("bar.sync 1, 128;" ::: "memory");
+        wait_for_previous();
         const int64_t hw = (int64_t)a.Ho * a.Wo;
         const int r = TW == 64 ? warp >> 1 : warp, px = TW == 64 ? (warp & 1) * 32 + lane : lane;
         Cursor at(a.ntiles, a.ntx, a.nty);
@@ -718,6 +728,7 @@ struct WgradArgs {
     int vecg;
     float *gw, *gb;          // gb nullable
     int ntx, nty, ntiles, NT, nmb;
+    bool chain;
     unsigned *err;
 };
 
@@ -753,6 +764,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
         sh.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    let_next_start();
     tc_before();
     __syncthreads();
     tc_after();
@@ -820,6 +832,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
             at.next(ngrp);
             return true;
         };
+        wait_for_previous();
 #pragma unroll
         for (int d = 0; d < D; ++d) load(q[d]);
         if constexpr (D == 1) {
@@ -863,6 +876,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
             bar_wait(&sh.empty[(n - 1) & 1], ((n - 1) >> 1) & 1, &none);
         }
     } else if (bar_wait(&sh.done, 0, abort)) {
+        wait_for_previous();
         tc_after();
         for (int mb = 0; mb < a.nmb; ++mb) {
             const int krow = mb * 128 + warp * 32 + lane;
@@ -881,6 +895,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
     __syncthreads();
     if (tid == 0 && sh.abort) atomicExch(a.err, 1u);
     if (warp == 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
+}
+
+template <typename... P, typename A>
+bool launch_chained(void (*fn)(P...), unsigned grid, int smem, cudaStream_t st, bool chain, const A &a)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chain ? 1 : 0;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, fn, a) == cudaSuccess;
 }
 
 // Dynamic shared memory above the default, once per kernel and device.
@@ -923,9 +954,7 @@ bool launch_conv(ConvArgs &a, int N, cudaStream_t st)
     a.ntiles = (int)nt;
     const int smem = 1024 + kSlots * 2 * kBlk + a.NT * a.KT * 2;
     if (!opt_in(k_conv_tile<M, TW, VEC>, kConvSmem, done)) return false;
-    count_launch();
-    k_conv_tile<M, TW, VEC><<<(unsigned)(nt < sm_count() ? nt : sm_count()), kThreads, smem, st>>>(a);
-    return true;
+    return launch_chained(k_conv_tile<M, TW, VEC>, (unsigned)(nt < sm_count() ? nt : sm_count()), smem, st, a.chain, a);
 }
 
 template <int M>
@@ -948,9 +977,7 @@ bool launch_wgrad_t(WgradArgs &a, int N, cudaStream_t st)
     a.ntiles = (int)nt;
     const int smem = 1024 + 2 * (a.nmb * 128 * 128 + a.NT * 128);
     if (!opt_in(k_wgrad_tile<M, TW, VEC>, kWgradSmem, done)) return false;
-    count_launch();
-    k_wgrad_tile<M, TW, VEC><<<(unsigned)(nt < sm_count() ? nt : sm_count()), kThreads, smem, st>>>(a);
-    return true;
+    return launch_chained(k_wgrad_tile<M, TW, VEC>, (unsigned)(nt < sm_count() ? nt : sm_count()), smem, st, a.chain, a);
 }
 
 template <int M>
@@ -968,9 +995,11 @@ int n_tile(int channels) { return channels <= 16 ? 16 : channels <= 32 ? 32 : 64
 bool conv_tile_fits(int Cin, int Cout) { return Cin >= 1 && Cin <= kMaxCh && Cout >= 1 && Cout <= kMaxCh; }
 
 bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
-               const float *bias, int Cout, int Ho, int Wo, int relu, const ConvOut &o, unsigned *err, cudaStream_t st)
+               const float *bias, int Cout, int Ho, int Wo, int relu, const ConvOut &o, unsigned *err, cudaStream_t st,
+               bool chain)
 {
     ConvArgs a{};
+    a.chain = chain;
     a.in = in;
     a.Cin = Cin;
     a.Hs = Hs;
@@ -992,9 +1021,10 @@ bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int H
 }
 
 bool wgrad_tile(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
-                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st)
+                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st, bool chain)
 {
     WgradArgs a{};
+    a.chain = chain;
     a.x = x;
     a.Cin = Cin;
     a.Hs = Hs;

@@ -314,6 +314,8 @@ void hess_backsolve(const HessState &hs, int j, cudaStream_t st);
 //   input gradient: v = gradient + add (nullable); out2 (nullable) = v; out = v where
 //   mask (nullable) > 0, else 0.  pool: v is first summed over 2 x 2 blocks (even Ho,
 //   Wo; the adjoint of nearest upsampling); no add or out2.
+// chain: the launch may start its set-up, the weights included, before the launch
+// preceding it on st has ended; only where that one is one of these kernels too.
 struct ConvOut {
     float *out = nullptr, *out2 = nullptr;
     const float *add = nullptr, *mask = nullptr;
@@ -323,10 +325,11 @@ bool conv_tile_fits(int Cin, int Cout);
 // grad = false: in [N][Cin][Hs][Ws] -> [N][Cout][Ho][Wo], weights W [Cout][Cin][3][3];
 // grad = true: in the output gradient, weights W [Cin][Cout][3][3].
 bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
-               const float *bias, int Cout, int Ho, int Wo, int relu, const ConvOut &o, unsigned *err, cudaStream_t st);
+               const float *bias, int Cout, int Ho, int Wo, int relu, const ConvOut &o, unsigned *err, cudaStream_t st,
+               bool chain = false);
 // Adds the weight gradient to gw (and the sums of g per channel to gb, nullable).
 bool wgrad_tile(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
-                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st);
+                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st, bool chain = false);
 
 // Learned stage: z = network(v) on a 2D grid (n0 x n1), see cnn.cu.
 mxp_status cnn_apply_vector(mxp_cnn *net, int n0, int n1, const double2 *v, double vnorm,
