@@ -165,10 +165,12 @@ def _check(status):
 
 
 def _ptr(t):
+    """Address of a vector.  A plain int: ctypes converts it to the pointer argument
+    without a c_void_p object, which counts where a call is one small launch."""
     import torch
-    if not (t.is_cuda and t.dtype == torch.complex128 and t.is_contiguous()):
+    if not (t.is_cuda and t.dtype is torch.complex128 and t.is_contiguous()):
         raise ValueError("vectors must be contiguous complex128 CUDA tensors")
-    return ct.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream_handle(stream):
@@ -374,11 +376,16 @@ class Problem:
     # -- operations (all on the problem's stream)
     def empty(self):
         import torch
-        return torch.empty(self.n_total, dtype=torch.complex128, device=f"cuda:{self.device}")
+        dev = self.__dict__.get("_torch_device")
+        if dev is None:                     # parsing the device's name takes longer than the allocation
+            dev = self._torch_device = torch.device("cuda", self.device)
+        return torch.empty(self.n_total, dtype=torch.complex128, device=dev)
 
     def apply_operator(self, x, shifted=False, out=None):
         y = self.empty() if out is None else out
-        _check(self._lib.mxp_apply_operator(self._h, int(bool(shifted)), _ptr(x), _ptr(y)))
+        s = self._lib.mxp_apply_operator(self._h, 1 if shifted else 0, _ptr(x), _ptr(y))
+        if s:
+            _check(s)
         return y
 
     def apply_phi(self, which, x, out=None):
@@ -542,8 +549,8 @@ def solve_batch(problems, prob_of_rhs, bs, xs, rtol=1e-6, restart=30, maxit=500)
     nprob, nrhs = len(problems), len(bs)
     hp = (ct.c_void_p * nprob)(*[p._h for p in problems])
     po = (ct.c_int * nrhs)(*prob_of_rhs)
-    bp = (ct.c_void_p * nrhs)(*[_ptr(b).value for b in bs])
-    xp = (ct.c_void_p * nrhs)(*[_ptr(x).value for x in xs])
+    bp = (ct.c_void_p * nrhs)(*[_ptr(b) for b in bs])
+    xp = (ct.c_void_p * nrhs)(*[_ptr(x) for x in xs])
     o = SolveOpts(rtol, restart, maxit, 0)
     st = (SolveStats * max(nrhs, 1))()
     s = lib.mxp_solve_batch(hp, nprob, nrhs, po, bp, xp, ct.byref(o), st)
