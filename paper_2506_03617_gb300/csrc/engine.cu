@@ -1029,6 +1029,11 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
         return passes;
     }
     const bool two = tm && which == 0 && tma3_two(P);
+    // psi_1 in complex128: u_{j+1} = p(X) u_j + xi_j w over the sub-steps, p the Taylor
+    // polynomial, xi_j the augmented scalar and w = u_1 (the first sub-step from u_0 = 0),
+    // which is what the augmented recursion computes; so after the first sub-step only
+    // the last sweep of a sub-step has a source (4 FP64 instructions a point saved).
+    const bool voc = sizeof(S) > 8 && which == 1 && Ssub > 1;
     for (int sub = 0; sub < Ssub; ++sub) {
         int in = iy;
         aug.begin_substep();
@@ -1037,11 +1042,12 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
             StepScalars<C> s1 = sc;              // first of two steps
             for (int s = 0; s < steps; ++s, --k) {
                 sc.sigma = PrecData<S>::c(cd(0.0, t / ((double)Ssub * k)));
-                sc.gamma = PrecData<S>::c(aug.gamma(k));
+                sc.gamma = PrecData<S>::c(voc && sub > 0 ? aug.z1 : aug.gamma(k));
                 sc.rho = PrecData<S>::c((sub == Ssub - 1 && k == 1) ? final_rho : cd(1.0));
                 aug.step(k);
                 if (s == 0) s1 = sc;
             }
+            const bool source = which && (!voc || sub == 0 || k == 0);      // k: steps left
             const int o = (in == iy) ? (iy + 1) % 3 : 3 - iy - in;
             if constexpr (sizeof(S) <= 8) {
                 cudaError_t ce = cudaSuccess;
@@ -1061,12 +1067,13 @@ static int64_t phi_action(mxp_problem *P, int which, const double2 *x, double2 *
                     return -1;
                 }
             }
-            if (!tm) sweep<S>(P, sc, b[in], b[iy], which ? vs : nullptr, b[o], st, passes > 0);
+            if (!tm) sweep<S>(P, sc, b[in], b[iy], source ? vs : nullptr, b[o], st, passes > 0 && !(voc && passes == m));
             in = o;
             passes += steps;
         }
         iy = in;
         aug.end_substep();
+        if (voc && sub == 0) cudaMemcpyAsync(vs, b[iy], (size_t)n * sizeof(S), cudaMemcpyDeviceToDevice, st);
     }
     if constexpr (sizeof(S) <= 8) {
         if (pitch != n0) launch_convert_out_rows<S>(b[iy], out, x, out_mode, n0, nrow, pitch, st);
