@@ -14,10 +14,10 @@
 // type, as it is between launches of single steps: the results are those of the
 // single-step sweeps to the last bit.
 //
-// Measured on 288^3, complex64: 203 us for two steps (230 us in single steps; 28 B a
+// Measured on 288^3, complex64: 200 us for two steps (230 us in single steps; 28 B a
 // point and two steps would be 98 us of HBM), about 65% of the issue slots in use; the
-// exp action 158 ms, before 180 ms.  On 129 x 102 x 115, in L2: 12.5 us a step, before
-// 14.4 us.
+// exp action 156 ms, before 180 ms.  In L2: 11.4 us a step of 129 x 102 x 115, before
+// 14.4 us; 24.5 us of 160^3, before 28.7 us; 3.2 us of 56^3, before 10.3 us.
 //
 // The kernel is bound by its instructions, so a warp's row takes one of three bodies:
 // all of it outside the PML (neighbours summed, real coefficient), in the PML in x
@@ -257,7 +257,8 @@ __global__ void __launch_bounds__(kThreads2, 2) k_step3z2(Geom g, const float2 *
     int cur = G::STAGE, nxt = 2 * G::STAGE;      // byte offsets of the stages of planes z and z + 1
     unsigned nbar = 2 % kRing, npar = 0;         // barrier and parity of plane z + 1
     int qcur = kRows * RX;                       // q(z) goes to qb + qcur, q(z - 1) is at the other half
-#pragma unroll 1
+    // twice: half of the register moves of the march (160^3: 24.5 us a step, rolled 27.1 us)
+#pragma unroll 2
     for (int z = z0 - 1; z <= z1 && !fail; ++z) {
         ok = mbar_wait(&bar[nbar], npar);
         const S *ps = reinterpret_cast<const S *>(stg + cur) + own0, *pn = reinterpret_cast<const S *>(stg + nxt) + own0;
