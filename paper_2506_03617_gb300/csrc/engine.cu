@@ -2332,7 +2332,11 @@ mxp_status mxp_horner_step(mxp_problem *P, const double *sigma, const double *ga
     sc.gamma = v_dev ? make_double2(gamma[0], gamma[1]) : make_double2(0.0, 0.0);
     sc.rho = make_double2(rho[0], rho[1]);
     set_faces<double2>(P, sc);
-    launch_step64(P->geom, P->coef64, P->kappa64, P->diag_ok ? P->diag64 : nullptr, sc, (const double2 *)p_dev,
+    // a captured step keeps the mu and shift of its capture: it forms its diagonal itself
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(P->stream, &cap);
+    const bool table = P->diag_ok && cap == cudaStreamCaptureStatusNone;
+    launch_step64(P->geom, P->coef64, P->kappa64, table ? P->diag64 : nullptr, sc, (const double2 *)p_dev,
                   (const double2 *)y_dev, (const double2 *)v_dev, (double2 *)out_dev, P->stream, false);
     P->passes += 1;
     CK(cudaGetLastError());

@@ -14,7 +14,7 @@
 // the general form needs 32 (3D: 42); an axis in its PML adds 4 to 6.
 // Measured: 28.0 us a sweep of 1088^2 unknowns (42 G updates/s; 12 instructions at
 // the measured 0.527 T/s would be 27 us), the general form 117 us; 3.5 us a sweep of
-// 160^2, before 8.2 us; the psi_1 action on 128^3 152 ms, before 477 ms.
+// 160^2, before 8.2 us; the psi_1 action on 128^3 127 ms, before 477 ms.
 #include "mxp_internal.h"
 
 namespace mxp {
