@@ -96,6 +96,7 @@ struct mxp_problem {
     double *kappa64 = nullptr;
     float *kappa32 = nullptr;
     double2 *coef64 = nullptr;            // coefficient table times h^2
+    double2 *coef64u = nullptr;           // the table itself (operator beside low-precision actions)
     double2 *diag64 = nullptr;            // scaled diagonal of the complex128 actions (ensure_diag)
     bool diag_ok = false;                 // diag64 belongs to the current parameters and faces
     float2 *coef32 = nullptr;
@@ -113,6 +114,7 @@ struct mxp_problem {
     int tma3_prec = -1;                  // precision the maps (or their absence) belong to
     float *kappa_pad = nullptr;          // kappa32 with padded rows, when n0 is no multiple of 4
     bool kappa_pad_ok = false;
+    bool lean = false;                   // device memory ran out: no diag64 and no kappa_pad
     std::vector<double2> coef_host;   // [3][3][nmax]
     // shift and plans
     double mu = 0;
@@ -321,16 +323,26 @@ static mxp_status upload_coef32(mxp_problem *P)
     return MXP_OK;
 }
 
+// The complex128 sweeps' table: coef_host times h^2.  Apart from upload_coefs so that
+// the compiler inlines and contracts build_coef_host there as it always has: other last
+// bits of the coefficients are differences of up to 5e-9 in a complex64 solve's solution.
+static __attribute__((noinline)) mxp_status upload_scaled64(mxp_problem *P)
+{
+    const double h2 = P->grid.h * P->grid.h;
+    P->kappa_pad_ok = false;
+    std::vector<double2> c64(P->coef_host);
+    for (double2 &c : c64) c = make_double2(c.x * h2, c.y * h2);
+    CK(cudaMemcpyAsync(P->coef64, c64.data(), c64.size() * sizeof(double2), cudaMemcpyHostToDevice, P->stream));
+    CK(cudaStreamSynchronize(P->stream));
+    return MXP_OK;
+}
+
 static mxp_status upload_coefs(mxp_problem *P)
 {
     build_coef_host(P);
     const size_t cnt = P->coef_host.size();
-    const double h2 = P->grid.h * P->grid.h;
-    std::vector<double2> c64(cnt);
-    for (size_t i = 0; i < cnt; ++i) c64[i] = make_double2(P->coef_host[i].x * h2, P->coef_host[i].y * h2);
-    CK(cudaMemcpyAsync(P->coef64, c64.data(), cnt * sizeof(double2), cudaMemcpyHostToDevice, P->stream));
+    CK(cudaMemcpyAsync(P->coef64u, P->coef_host.data(), cnt * sizeof(double2), cudaMemcpyHostToDevice, P->stream));
     compute_kappa(P->c_dev, P->prm.omega, P->kappa64, P->kappa32, P->ntot, P->stream);
-    P->kappa_pad_ok = false;
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(P->stream));
     return MXP_OK;
@@ -367,13 +379,46 @@ static void free_arnoldi(Arnoldi &a)
     a = Arnoldi{};
 }
 
+static void clear_graphs(mxp_problem *P);
+
+// Device memory for vectors of the problem.  Where none is left, the tables that only
+// save time are given back and the sweeps do without them (the same results: diag_of
+// per point, the register-marching 3D sweep).
+template <typename T>
+static cudaError_t dev_alloc(mxp_problem *P, T **p, size_t bytes)
+{
+    const cudaError_t e = cudaMalloc((void **)p, bytes);
+    if (e != cudaErrorMemoryAllocation || P->lean || (!P->diag64 && !P->kappa_pad)) return e;
+    cudaGetLastError();
+    cudaStreamSynchronize(P->stream);
+    clear_graphs(P);
+    cudaFree(P->diag64);
+    P->diag64 = nullptr;
+    P->diag_ok = false;
+    if (P->kappa_pad) {
+        tma3_destroy(P->tma3);
+        P->tma3 = nullptr;
+        cudaFree(P->kappa_pad);
+        P->kappa_pad = nullptr;
+    }
+    P->lean = true;
+    return cudaMalloc((void **)p, bytes);
+}
+
+static bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &cap);
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 static mxp_status ensure_arnoldi(mxp_problem *P, Arnoldi &a, int R, bool flexible)
 {
     if (a.V && a.R >= R && (!flexible || a.Z)) return MXP_OK;
     free_arnoldi(a);
     const int64_t n = P->ntot;
-    CK(cudaMalloc(&a.V, (size_t)(R + 1) * n * sizeof(double2)));
-    if (flexible) CK(cudaMalloc(&a.Z, (size_t)R * n * sizeof(double2)));
+    CK(dev_alloc(P, &a.V, (size_t)(R + 1) * n * sizeof(double2)));
+    if (flexible) CK(dev_alloc(P, &a.Z, (size_t)R * n * sizeof(double2)));
     CK(cudaMalloc(&a.hs.H, (size_t)(R + 1) * R * sizeof(double2)));
     CK(cudaMalloc(&a.hs.cs, R * sizeof(double)));
     CK(cudaMalloc(&a.hs.sn, R * sizeof(double2)));
@@ -394,10 +439,10 @@ static mxp_status ensure_base(mxp_problem *P)
     const int64_t n = P->ntot;
     if (P->prm.prec == MXP_C128) CKS(ensure_diag(P));
     for (int i = 0; i < 4; ++i)
-        if (!P->hb[i]) CK(cudaMalloc(&P->hb[i], (size_t)n * 16));
-    if (!P->rt) CK(cudaMalloc(&P->rt, n * sizeof(double2)));
-    if (!P->tmp) CK(cudaMalloc(&P->tmp, n * sizeof(double2)));
-    if (!P->tmp2) CK(cudaMalloc(&P->tmp2, n * sizeof(double2)));
+        if (!P->hb[i]) CK(dev_alloc(P, &P->hb[i], (size_t)n * 16));
+    if (!P->rt) CK(dev_alloc(P, &P->rt, n * sizeof(double2)));
+    if (!P->tmp) CK(dev_alloc(P, &P->tmp, n * sizeof(double2)));
+    if (!P->tmp2) CK(dev_alloc(P, &P->tmp2, n * sizeof(double2)));
     if (!P->ks.partials) {
         P->ks.grid = sm_count() * 4;
         CK(cudaMalloc(&P->ks.partials, (size_t)P->ks.grid * kChunk * sizeof(double2)));
@@ -454,11 +499,17 @@ template <> struct PrecData<__nv_bfloat162> : PrecData<float2> {};
 
 // The scaled diagonal of the complex128 actions: made before the first action
 // after a change of parameters or faces (a slab's at its set-up: mxp_horner_step
-// neither allocates nor launches more than its sweep).
+// neither allocates nor launches more than its sweep).  Without it (no memory left, or
+// inside a capture, where nothing is made yet) the sweeps form it per point.
 static mxp_status ensure_diag(mxp_problem *P)
 {
-    if (P->diag_ok) return MXP_OK;
-    if (!P->diag64) CK(cudaMalloc(&P->diag64, (size_t)P->ntot * sizeof(double2)));
+    if (P->diag_ok || P->lean || capturing(P->stream)) return MXP_OK;
+    if (!P->diag64 && cudaMalloc(&P->diag64, (size_t)P->ntot * sizeof(double2)) != cudaSuccess) {
+        cudaGetLastError();
+        P->diag64 = nullptr;
+        P->lean = true;
+        return MXP_OK;
+    }
     StepScalars<double2> sc{};
     sc.zfac = make_double2(1.0, P->prm.shift_s);
     sc.mu = P->mu;
@@ -476,7 +527,7 @@ static void sweep(mxp_problem *P, const StepScalars<typename St<S>::C> &sc, cons
                   S *pout, cudaStream_t st, bool chain)
 {
     if constexpr (sizeof(S) == sizeof(double2))
-        launch_step64(P->geom, P->coef64, P->kappa64, P->diag64, sc, pin, y, v, pout, st, chain);
+        launch_step64(P->geom, P->coef64, P->kappa64, P->diag_ok ? P->diag64 : nullptr, sc, pin, y, v, pout, st, chain);
     else
         launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc, pin, y, v, pout, st);
 }
@@ -837,9 +888,10 @@ static const Tma3Maps *tma3_maps(mxp_problem *P, bool padded)
 {
     if (P->grid.dim != 3 || P->nfaces) return nullptr;
     const int n0 = P->geom.n[0], pitch = tma3_pitch(P->geom);
-    if (pitch != n0 && !padded) return nullptr;
+    if (pitch != n0 && (!padded || P->lean)) return nullptr;
     const int64_t rows = (int64_t)P->geom.n[1] * P->geom.n[2];
     if (pitch > n0 && !P->kappa_pad_ok) {
+        if (capturing(P->stream)) return nullptr;
         if (!P->kappa_pad && cudaMalloc(&P->kappa_pad, (size_t)rows * pitch * sizeof(float)) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
@@ -1101,7 +1153,14 @@ static void apply_op(mxp_problem *P, int shifted, const double2 *x, double2 *y, 
     sc.gamma = make_double2(0.0, 0.0);
     sc.rho = make_double2(1.0, 0.0);
     set_faces<double2>(P, sc);
-    launch_step64(P->geom, P->coef64, P->kappa64, nullptr, sc, x, nullptr, nullptr, y, st ? st : P->stream, false);
+    // Beside complex64 / bf16 actions the operator keeps its plain form: the vectors of a
+    // solve are rounded to the actions' type, which turns another order of the operator's
+    // additions (1e-16) into differences of 1e-9 to 1e-8 in the solution.  It is one of
+    // thousands of sweeps there (114 us against 55 us a launch on 1088^2).
+    if (P->prm.prec != MXP_C128)
+        launch_operator(P->geom, P->coef64u, P->kappa64, sc, x, y, st ? st : P->stream);
+    else
+        launch_step64(P->geom, P->coef64, P->kappa64, nullptr, sc, x, nullptr, nullptr, y, st ? st : P->stream, false);
     P->passes += 1;
 }
 
@@ -1379,7 +1438,7 @@ static mxp_status ensure_batch(mxp_problem *P, int nr, int Rout, int Rin)
         for (int i = 0; i < 4; ++i) { cudaFree(P->bslot[i]); P->bslot[i] = nullptr; }
         if (P->bhost) cudaFreeHost(P->bhost);
         P->bhost = nullptr;
-        for (int i = 0; i < 4; ++i) CK(cudaMalloc(&P->bslot[i], (size_t)nr * n * 16));
+        for (int i = 0; i < 4; ++i) CK(dev_alloc(P, &P->bslot[i], (size_t)nr * n * 16));
         CK(cudaMallocHost(&P->bhost, (size_t)nr * 8 * sizeof(double)));
         P->bcap = nr;
     }
@@ -1388,8 +1447,8 @@ static mxp_status ensure_batch(mxp_problem *P, int nr, int Rout, int Rin)
         auto &s = P->rhs[r];
         CKS(ensure_arnoldi(P, s.outer, Rout, true));
         CKS(ensure_arnoldi(P, s.inner, Rin, false));
-        if (!s.rt) CK(cudaMalloc(&s.rt, n * sizeof(double2)));
-        if (!s.r) CK(cudaMalloc(&s.r, n * sizeof(double2)));
+        if (!s.rt) CK(dev_alloc(P, &s.rt, n * sizeof(double2)));
+        if (!s.r) CK(dev_alloc(P, &s.r, n * sizeof(double2)));
     }
     return MXP_OK;
 }
@@ -2289,12 +2348,14 @@ static mxp_status create_impl(const mxp_grid *grid, int64_t row0, int64_t nrows,
         cudaMalloc(&P->kappa64, ntot * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&P->kappa32, ntot * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&P->coef64, cnt * sizeof(double2)) != cudaSuccess ||
+        cudaMalloc(&P->coef64u, cnt * sizeof(double2)) != cudaSuccess ||
         cudaMalloc(&P->coef32, cnt * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&P->coef32s, cnt * sizeof(float2)) != cudaSuccess)
         return bail(fail(MXP_ENOMEM, "device allocation failed"));
     if (cudaMemcpyAsync(P->c_dev, c_host, ntot * sizeof(double), cudaMemcpyHostToDevice, P->stream) != cudaSuccess)
         return bail(fail(MXP_ECUDA, "copy of the medium failed"));
     mxp_status s = upload_coefs(P);
+    if (s == MXP_OK) s = upload_scaled64(P);
     if (s != MXP_OK) return bail(s);
     update_plans(P);
     s = upload_coef32(P);
@@ -2333,9 +2394,7 @@ mxp_status mxp_horner_step(mxp_problem *P, const double *sigma, const double *ga
     sc.rho = make_double2(rho[0], rho[1]);
     set_faces<double2>(P, sc);
     // a captured step keeps the mu and shift of its capture: it forms its diagonal itself
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(P->stream, &cap);
-    const bool table = P->diag_ok && cap == cudaStreamCaptureStatusNone;
+    const bool table = P->diag_ok && !capturing(P->stream);
     launch_step64(P->geom, P->coef64, P->kappa64, table ? P->diag64 : nullptr, sc, (const double2 *)p_dev,
                   (const double2 *)y_dev, (const double2 *)v_dev, (double2 *)out_dev, P->stream, false);
     P->passes += 1;
@@ -2526,7 +2585,10 @@ mxp_status mxp_set_params(mxp_problem *P, const mxp_params *p)
     DeviceGuard guard(P->device);
     const bool recoef = np.omega != P->prm.omega || np.c_pml != P->prm.c_pml;
     P->prm = np;
-    if (recoef) CKS(upload_coefs(P));
+    if (recoef) {
+        CKS(upload_coefs(P));
+        CKS(upload_scaled64(P));
+    }
     if (recoef && P->nfaces) CKS(build_faces(P));
     update_plans(P);
     CKS(upload_coef32(P));
@@ -2670,8 +2732,8 @@ mxp_status mxp_solve_host(mxp_problem *P, const void *b_host, void *x_host, cons
     CKS(check_opts(opts));
     DeviceGuard guard(P->device);
     const size_t bytes = (size_t)P->ntot * sizeof(double2);
-    if (!P->bdev) CK(cudaMalloc(&P->bdev, bytes));
-    if (!P->xdev) CK(cudaMalloc(&P->xdev, bytes));
+    if (!P->bdev) CK(dev_alloc(P, &P->bdev, bytes));
+    if (!P->xdev) CK(dev_alloc(P, &P->xdev, bytes));
     CK(cudaMemcpyAsync(P->bdev, b_host, bytes, cudaMemcpyHostToDevice, P->stream));
     if (opts->x0_given) CK(cudaMemcpyAsync(P->xdev, x_host, bytes, cudaMemcpyHostToDevice, P->stream));
     mxp_status s = fgmres_solve(P, P->bdev, P->xdev, opts, st);
@@ -2821,7 +2883,7 @@ void mxp_destroy(mxp_problem *P)
     DeviceGuard guard(P->device);
     cudaStreamSynchronize(P->stream);
     cudaFree(P->c_dev); cudaFree(P->kappa64); cudaFree(P->kappa32);
-    cudaFree(P->coef64); cudaFree(P->diag64); cudaFree(P->coef32); cudaFree(P->coef32s);
+    cudaFree(P->coef64); cudaFree(P->coef64u); cudaFree(P->diag64); cudaFree(P->coef32); cudaFree(P->coef32s);
     cudaFree(P->face64); cudaFree(P->face32); cudaFree(P->face32s);
     for (int i = 0; i < 4; ++i) cudaFree(P->hb[i]);
     tma3_destroy(P->tma3);

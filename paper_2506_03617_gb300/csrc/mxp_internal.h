@@ -87,7 +87,7 @@ template <> struct CT<double2> { using R = double; static __host__ __device__ do
 template <> struct CT<float2> { using R = float; static __host__ __device__ float2 mk(float a, float b) { return make_float2(a, b); } };
 
 // ---------------------------------------------------------------- geometry
-struct Geom {
+struct GeomBase {
     int dim;
     int n[3];          // unknowns per axis (1 for unused axes)
     int64_t s1, s2;    // strides of axes 1 and 2
@@ -96,6 +96,8 @@ struct Geom {
     int fast = 0;      // 1: unknowns outside the PML use the real interior coefficient ih2
     int npml = 0;
     double ih2 = 0;    // 1 / h^2
+};
+struct Geom : GeomBase {
     // positions [in_lo, in_hi) of each axis lie outside its PML: their neighbour
     // coefficients are the real 1 / h^2 (complex128 sweeps)
     int in_lo[3] = {0, 0, 0}, in_hi[3] = {1, 1, 1};
@@ -146,6 +148,11 @@ template <typename S>
 void launch_step(const Geom &g, const typename St<S>::C *coef, const typename St<S>::R *kappa,
                  const StepScalars<typename St<S>::C> &sc, const S *pin, const S *y, const S *v,
                  S *pout, cudaStream_t st);
+
+// y = rho sigma A x in complex128 with the unscaled table: the operator of problems
+// whose actions run in complex64 or bf16 storage.
+void launch_operator(const Geom &g, const double2 *coef, const double *kappa, const StepScalars<double2> &sc,
+                     const double2 *x, double2 *y, cudaStream_t st);
 
 // The same step in complex128 (stencil64.cu); coef is the table times h^2.  diag
 // (nullable): the sweep's scaled diagonal from make_diag64, formed per point

@@ -1,6 +1,6 @@
 // Stencil kernels: one Taylor-Horner step of the exponential-integrator actions
 // (Def. psi) for complex64 and bfloat16-storage vectors (complex128: stencil64.cu),
-// and the conversions between the stored types.
+// the operator beside such actions, and the conversions between the stored types.
 //
 // Operator (Eq. helmholtz with the stretched Laplacian of Eq. pml-1d-s on each
 // axis, shift of Sec. 3.4), written with the per-axis coefficient table
@@ -35,7 +35,7 @@ __device__ __forceinline__ C czero() { return CT<C>::mk(0, 0); }
 // out = rho * ( y + sigma * ((A_s - mu) p) + gamma * v )
 // HAS_Y = false drops y; HAS_V = false drops v.
 template <typename S, int DIM, bool HAS_Y, bool HAS_V>
-__global__ void __launch_bounds__(128) k_step(Geom g, const typename St<S>::C *__restrict__ coef,
+__global__ void __launch_bounds__(128) k_step(GeomBase g, const typename St<S>::C *__restrict__ coef,
                                               const typename St<S>::R *__restrict__ kappa,
                                               StepScalars<typename St<S>::C> sc,
                                               const S *__restrict__ pin, const S *__restrict__ y,
@@ -219,6 +219,16 @@ void launch_step(const Geom &g, const typename St<S>::C *coef, const typename St
     if (g.dim == 3 && sc.nfaces == 0) launch_step3z<S>(g, coef, kappa, sc, pin, y, v, pout, st);
     else if (g.dim == 3) launch_step_dim<S, 3>(g, coef, kappa, sc, pin, y, v, pout, st);
     else launch_step_dim<S, 2>(g, coef, kappa, sc, pin, y, v, pout, st);
+}
+
+void launch_operator(const Geom &g, const double2 *coef, const double *kappa, const StepScalars<double2> &sc,
+                     const double2 *x, double2 *y, cudaStream_t st)
+{
+    dim3 block(128);
+    dim3 grid((g.n[0] + 127) / 128, g.n[1], g.n[2]);
+    count_launch();
+    if (g.dim == 3) k_step<double2, 3, false, false><<<grid, block, 0, st>>>(g, coef, kappa, sc, x, nullptr, nullptr, y);
+    else k_step<double2, 2, false, false><<<grid, block, 0, st>>>(g, coef, kappa, sc, x, nullptr, nullptr, y);
 }
 
 // ---------------------------------------------------------------- conversions

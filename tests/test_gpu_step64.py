@@ -63,6 +63,22 @@ def test_horner_step(native, ni, npml, bc, prec):
         assert np.max(np.abs(out - ref)) <= 1e-13 * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("ni,npml,bc", CASES, ids=[f"{c[0]}-{c[1]}" for c in CASES])
+def test_operator_forms(native, ni, npml, bc):
+    """The operator of a complex128 problem and the one beside low-precision actions."""
+    g, c, p, codes, (x, _, _) = _setup(ni, npml, bc)
+    O = oracle.Problem.from_grid(g, c, p, bc=codes)
+    G = native.Problem.from_grid(g, c, p)
+    if bc:
+        G.set_boundary(bc)
+    xd = torch.from_numpy(x).cuda()
+    for prec in ("c128", "c64", "bf16s"):
+        G.set_params(prec=prec)
+        for shifted in (False, True):
+            out, ref = G.apply_operator(xd, shifted=shifted).cpu().numpy(), O.apply(x, shifted=shifted)
+            assert np.max(np.abs(out - ref)) <= 1e-13 * np.max(np.abs(ref))
+
+
 @pytest.mark.parametrize("dim", [2, 3])
 def test_slab_rows(native, dim):
     ni = (37, 30) if dim == 2 else (9, 8, 26)
