@@ -582,7 +582,9 @@ def run_ours(args):
                                    "alg_tflops": fl64, "dfma_peak_tflops": fp64_peak,
                                    "frac_of_dfma_peak": fl64 / fp64_peak,
                                    "roofline_note": "FP64 sweeps on an L2-resident grid: bound by "
-                                                    "the FP64 pipe (measured DFMA throughput, of measured)",
+                                                    "the FP64 pipe (measured DFMA throughput, of measured); "
+                                                    "alg_tflops counts 24 flops per interior update, the "
+                                                    "sweep issues 12 FP64 instructions for them",
                                    "speedup_of_this_precision": t64 / (total_max / args.steps),
                                    f"{args.prec}_solution_rel_err":
                                        float(torch.linalg.vector_norm(x_lo - x64)) / nrm64}
