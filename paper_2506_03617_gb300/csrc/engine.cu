@@ -449,7 +449,7 @@ static mxp_status ensure_base(mxp_problem *P)
     }
     if (!P->host_scal) CK(cudaMallocHost(&P->host_scal, 8 * sizeof(double)));
     if (!P->bar) {
-        // [0..3] grid-barrier words and error flag, [4..] per-tile pass epochs
+        // [0..3] grid-barrier words and error flag, from kPersistFlagStride per-tile pass epochs
         CK(cudaMalloc(&P->bar, kPersistBarWords * sizeof(unsigned)));
         CK(cudaMemsetAsync(P->bar, 0, kPersistBarWords * sizeof(unsigned), P->stream));
     }

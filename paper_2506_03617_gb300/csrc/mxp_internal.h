@@ -174,10 +174,15 @@ constexpr int kMaxFuse = 8;
 
 // Synchronisation words of the persistent exp kernel: [0] arrival count,
 // [1] generation, [2] error flag, [3] spare, then one epoch word per tile, each
-// in its own 32-byte sector (tiles poll their neighbours' words concurrently).
+// in its own 128-byte line.  Up to eight neighbours poll a word while its tile posts
+// to it; with four words to a line (a sector each) a post also meets the polls of
+// three other tiles, and how much that costs depends on where the line lies: psi_1 on
+// 544^2 in bf16 storage took 3.09 to 3.19 ms by the address of these words, an exp
+// action 2.93 ms on 1088^2 and 2.35 ms on 288^2 (complex64).  With a line each 2.84 to
+// 2.93, 2.75 and 2.11 ms (two words to a line 2.95, 2.79, 2.16; 256 bytes apart as 128).
 constexpr int kPersistMaxTiles = 4096;
-constexpr int kPersistFlagStride = 8;
-constexpr size_t kPersistBarWords = 4 + (size_t)kPersistMaxTiles * kPersistFlagStride;
+constexpr int kPersistFlagStride = 32;
+constexpr size_t kPersistBarWords = kPersistFlagStride + (size_t)kPersistMaxTiles * kPersistFlagStride;
 struct FusedStep {
     double tau, gamma_re, gamma_im, rho_re, rho_im;
     int rho_on;

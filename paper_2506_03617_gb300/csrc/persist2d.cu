@@ -31,7 +31,7 @@ struct PersistArgs {
     const float *tau;            // per step: tau / h^2 (operator scaled by h^2), npass * K
     int npass, pass_per_sub;     // passes in total and per sub-step
     float2 rho;                  // e^{i t mu}: multiplies the result (undoes the shift)
-    unsigned *bar;               // [0] arrival count, [1] generation, [2] error flag, [4..] tile epochs
+    unsigned *bar;               // [0] arrival count, [1] generation, [2] error flag, [kPersistFlagStride ..] tile epochs
     // psi_1 by sub-steps (nullptr for exp): after sub-step j (1-based) the tile
     // gains wcoef[j-1] * w (w in the storage type S)
     const void *w;
@@ -111,9 +111,9 @@ __device__ __forceinline__ bool neighbour_sync(unsigned *bar, int bx, int by, in
     if (entry_barrier) __syncthreads();
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        const unsigned *flags = bar + 4;
+        const unsigned *flags = bar + kPersistFlagStride;
         volatile unsigned *verr = bar + 2;
-        if (lane == 0) st_release_gpu(bar + 4 + (by * ntx + bx) * kPersistFlagStride, epoch);
+        if (lane == 0) st_release_gpu(bar + kPersistFlagStride + (by * ntx + bx) * kPersistFlagStride, epoch);
         int ok = 1;
         if (lane < 9 && lane != 4) {
             const int nx = bx + lane % 3 - 1, ny = by + lane / 3 - 1;
@@ -852,7 +852,7 @@ cudaError_t launch_persist2d(int id, const Geom &g, int npml, const float2 *coef
     // reads it (and a launch that finds it set leaves its pass loop at once)
     cudaError_t e = cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st);
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(bar + 4, 0, (size_t)ntx * nty * kPersistFlagStride * sizeof(unsigned), st);
+        e = cudaMemsetAsync(bar + kPersistFlagStride, 0, (size_t)ntx * nty * kPersistFlagStride * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     count_launch();
     if (a.nfaces && !c.faces) return cudaErrorInvalidValue;   // this configuration has no face terms
