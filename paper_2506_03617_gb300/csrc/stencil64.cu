@@ -13,7 +13,7 @@
 // then 6 additions + 4 + 2 multiply-adds = 12 FP64 instructions (3D: 16), where
 // the general form needs 32 (3D: 42); an axis in its PML adds 4 to 6.
 // Measured: 28.0 us a sweep of 1088^2 unknowns (42 G updates/s; 12 instructions at
-// the measured 0.527 T/s would be 27 us), the general form 117 us; 3.5 us a sweep of
+// the measured 0.527 T/s would be 27 us), the general form 117 us; 2.4 us a sweep of
 // 160^2, before 8.2 us; the psi_1 action on 128^3 127 ms, before 477 ms.
 #include "mxp_internal.h"
 
@@ -38,6 +38,9 @@ __device__ __forceinline__ double2 ldv(const double2 *p)
     asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(r.x), "=d"(r.y) : "l"(p) : "memory");
     return r;
 }
+
+// Lets the next sweep's blocks start; they wait for this sweep's end before they read.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <int DIM>
 __device__ __forceinline__ double2 face_terms(const Geom &g, const Scal64 &sc, int i, int j, int k)
@@ -83,7 +86,7 @@ __device__ __forceinline__ void fma_c(double2 &a, double2 c, double2 p)
 // the compiler to predicate, and a predicated-off FP64 instruction takes its 64
 // cycles of the pipe all the same (28 instructions a point were issued instead of
 // 14, 62.7 us a 1088^2 sweep).
-template <int DIM, bool HAS_Y, bool HAS_V, bool FAST, bool PX, bool PY, bool PZ>
+template <int DIM, bool HAS_Y, bool HAS_V, bool FAST, int REL, bool PX, bool PY, bool PZ>
 __device__ __forceinline__ void point64(const Geom &g, const double2 *__restrict__ coef,
                                         const double *__restrict__ kappa, const double2 *__restrict__ diag,
                                         const Scal64 &sc, const double2 *pin, const double2 *y, const double2 *v,
@@ -96,8 +99,9 @@ __device__ __forceinline__ void point64(const Geom &g, const double2 *__restrict
     if (PX) { wpx = coef[i]; wmx = coef[nm + i]; }
     if (PY) { wpy = coef[3 * nm + j]; wmy = coef[4 * nm + j]; }
     if (PZ) { wpz = coef[6 * nm + k]; wmz = coef[7 * nm + k]; }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (REL == 0) let_next_start();
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (REL == 1) let_next_start();
     const double2 zero = make_double2(0.0, 0.0);
     const double2 *pq = pin + q;
     const double2 pc = ldv(pq);
@@ -139,13 +143,15 @@ __device__ __forceinline__ void point64(const Geom &g, const double2 *__restrict
     }
     if (HAS_V) fma_c(o, sc.gam, vv);
     if (!FAST) o = cmul(sc.rho, o);
+    if (REL == 2) let_next_start();
     if (act) pout[q] = o;
 }
 
 // One point per thread, a warp along x (so the PML of y and z is uniform over a
 // warp, and a warp takes the general x form when any of its lanes needs it).
-// FAST: sigma imaginary and rho = 1 (every sweep of an action but the last).
-template <int DIM, bool HAS_Y, bool HAS_V, bool FAST>
+// FAST: sigma imaginary and rho = 1 (every sweep of an action but the last).  REL: see
+// released_at (a template argument: tested at run time it costs 0.2 us a sweep).
+template <int DIM, bool HAS_Y, bool HAS_V, bool FAST, int REL>
 __global__ void __launch_bounds__(256) k_step64(Geom g, const double2 *__restrict__ coef,
                                                 const double *__restrict__ kappa, const double2 *__restrict__ diag,
                                                 const __grid_constant__ Scal64 sc, const double2 *pin,
@@ -161,7 +167,7 @@ __global__ void __launch_bounds__(256) k_step64(Geom g, const double2 *__restric
     const bool py = jc < g.in_lo[1] || jc >= g.in_hi[1];
     const bool pz = DIM >= 3 && (k < g.in_lo[2] || k >= g.in_hi[2]);
 #define MXP_POINT(X, Y, Z) \
-    point64<DIM, HAS_Y, HAS_V, FAST, X, Y, Z>(g, coef, kappa, diag, sc, pin, y, v, pout, ic, jc, k, q, act)
+    point64<DIM, HAS_Y, HAS_V, FAST, REL, X, Y, Z>(g, coef, kappa, diag, sc, pin, y, v, pout, ic, jc, k, q, act)
     switch ((px ? 1 : 0) | (py ? 2 : 0) | (pz ? 4 : 0)) {
     case 0: MXP_POINT(false, false, false); break;
     case 1: MXP_POINT(true, false, false); break;
@@ -185,6 +191,23 @@ __global__ void __launch_bounds__(256) k_diag64(Geom g, const double2 *__restric
     if (i >= g.n[0] || j >= g.n[1]) return;
     const int64_t q = i + g.s1 * j + g.s2 * k;
     diag[q] = diag_of<DIM>(g, coef, kappa, sc, i, j, k, q);
+}
+
+// Where a sweep lets the next one start: before its own wait (0), after it (1) or before
+// its stores (2).  Released before the wait, a third and a fourth sweep start too while
+// the first still runs: waiting blocks fill the SMs, and those of a later sweep go
+// wherever some end, several to one SM and none to another (224^2: 6.3 us a sweep, 24^3
+// 5.4 us).  After the wait there is at most one sweep ahead, evenly placed as long as
+// two fit side by side (224^2 3.0, 24^3 2.6, but 352^2 7.2 us); before the stores it is
+// placed on SMs that are about to be free (3.0, 2.8 and 5.0 us).  Up to four warps an
+// SM the earlier start gains more; up to one, waiting blocks do no harm (24^2: 1.97,
+// 2.17 and 2.21 us).  From some forty warps an SM on a sweep does not fit the SMs at
+// once: its own blocks fill every gap, and the early release saves up to 3% (512^2: 8.2,
+// 8.2 and 8.45 us).
+static int released_at(const Geom &g)
+{
+    const int64_t warps = (int64_t)((g.n[0] + 31) / 32) * g.n[1] * g.n[2], sms = sm_count();
+    return warps <= sms || warps > 40 * sms ? 0 : warps <= 4 * sms ? 1 : 2;
 }
 
 static Scal64 scaled(const Geom &g, const StepScalars<double2> &s)
@@ -230,8 +253,21 @@ static void launch64(const Geom &g, const double2 *coef, const double *kappa, co
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = chain ? 1 : 0;
-    if (sc.fast) cudaLaunchKernelEx(&cfg, k_step64<DIM, Y, V, true>, g, coef, kappa, diag, sc, pin, y, v, pout);
-    else cudaLaunchKernelEx(&cfg, k_step64<DIM, Y, V, false>, g, coef, kappa, diag, sc, pin, y, v, pout);
+    // sweeps with y and the fast scalars are chained to one another; the others have
+    // nothing behind them that is (an operator, a single step) or come once an action
+    const int rel = Y && sc.fast ? released_at(g) : 2;
+    if constexpr (Y) {
+        if (rel == 0) {
+            cudaLaunchKernelEx(&cfg, k_step64<DIM, Y, V, true, 0>, g, coef, kappa, diag, sc, pin, y, v, pout);
+            return;
+        }
+        if (rel == 1) {
+            cudaLaunchKernelEx(&cfg, k_step64<DIM, Y, V, true, 1>, g, coef, kappa, diag, sc, pin, y, v, pout);
+            return;
+        }
+    }
+    if (sc.fast) cudaLaunchKernelEx(&cfg, k_step64<DIM, Y, V, true, 2>, g, coef, kappa, diag, sc, pin, y, v, pout);
+    else cudaLaunchKernelEx(&cfg, k_step64<DIM, Y, V, false, 2>, g, coef, kappa, diag, sc, pin, y, v, pout);
 }
 
 template <int DIM>
