@@ -227,13 +227,16 @@ static Scal64 scaled(const Geom &g, const StepScalars<double2> &s)
     return r;
 }
 
-// Rows per block: 8 (256 threads); fewer on grids too small to give every SM four
-// such blocks, so that the last wave is not one block of a whole SM's work.
+// Rows per block (a warp each): 4, one warp for each partition of an SM; 2 on grids
+// too small to give every SM four such blocks, so that the last wave is not one block of
+// a whole SM's work.  Blocks of 8 are no faster anywhere (us a sweep, 8 against 4 rows:
+// 512^2 8.2 and 8.0, 56^3 10.6 and 9.9, 1088^2 28.6 and 28.3), blocks of 1 run out of
+// block slots (1088^2 38, 320^2 5.1 against 4.5) and gain little on small grids (216^2
+// 3.3 against 2.9, 28^3 2.9 and 2.9).
 static void shape64(const Geom &g, dim3 *grid, dim3 *block)
 {
     const int64_t bx = (g.n[0] + 31) / 32;
-    int by = 8;
-    while (by > 2 && bx * ((g.n[1] + by - 1) / by) * g.n[2] < (int64_t)sm_count() * 4) by /= 2;
+    const int by = bx * ((g.n[1] + 3) / 4) * g.n[2] < (int64_t)sm_count() * 4 ? 2 : 4;
     *block = dim3(32, by);
     *grid = dim3((unsigned)bx, (g.n[1] + by - 1) / by, g.n[2]);
 }
