@@ -33,8 +33,8 @@
 // whatever N is (135 us), under the stores of A (150 us without the loads); the loads'
 // latency adds 40 us, the epilogue 8 us.  The weights and the launch cost 12 us a
 // kernel, which is most of a layer on a batch of 32 crops of 64 x 64; as dependent
-// launches they run under the kernel before (0.57 -> 0.52 ms for forward and gradients
-// of that batch, before these kernels 4.28 ms).  One forward pass on 1088^2: 0.70 ms,
+// launches they run under the kernel before (0.57 -> 0.51 ms for forward and gradients
+// of that batch, before these kernels 4.28 ms).  One forward pass on 1088^2: 0.68 ms,
 // before 2.98 ms.
 //
 // Every wait on an mbarrier is bounded; on timeout the kernel sets *err, all roles
@@ -110,8 +110,14 @@ __device__ __forceinline__ bool all_of_128(bool ok)
 
 // Programmatic dependent launch: the next kernel's set-up (barriers, tensor memory,
 // weights) may run under this kernel's last tiles; its activations wait for this one.
-__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// It is let go when this kernel no longer waits itself: before that, the CTAs of kernels
+// further on took SMs and shared memory from the next one's (forward pass on 30 x 34
+// 82 -> 71 us, on 1088^2 701 -> 676 us, with gradients on 32 crops of 64^2 545 -> 534 us).
+__device__ __forceinline__ void wait_for_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -507,7 +513,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
         for (int i = tid; i < kSlots * 2 * kBlk / 16; i += kThreads) reinterpret_cast<uint4 *>(sA)[i] = make_uint4(0, 0, 0, 0);
         fence_async_smem();
     }
-    let_next_start();
     tc_before();
     __syncthreads();
     tc_after();
@@ -764,7 +769,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
         sh.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    let_next_start();
     tc_before();
     __syncthreads();
     tc_after();

@@ -217,8 +217,11 @@ __global__ void __launch_bounds__(kThreads2, 2) k_step3z2(Geom g, const float2 *
             wxy[r][c] = add_rn(wcx[c], wcy);
         }
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the next launch starts when this one no longer waits: released before the wait, a
+    // third and a fourth would be resident too, unevenly spread (exp action on 24^3 3.66
+    // and 3.44 ms, 28 x 14 x 12 3.55 and 3.43, 160^3 42.3 and 41.9)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0)
         for (int pi = 0; pi < kRing && pi < nload; ++pi) issue(pi);
 
