@@ -327,12 +327,12 @@ typedef enum {
     MXP_SWEEP_FUSED_2D = 1,       /* K steps per launch on shared-memory tiles */
     MXP_SWEEP_PERSISTENT_2D = 2,  /* one cooperative launch per action, grid held on chip */
     MXP_SWEEP_FUSED_3D = 3,       /* K steps per launch by z-marching temporal blocking */
-    MXP_SWEEP_ZMARCH_3D = 4,      /* one launch per step, threads march along z in registers */
-    MXP_SWEEP_ZMARCH_TMA_3D = 5   /* one launch per step, planes staged by TMA (n0 % 4 == 0) */
+    MXP_SWEEP_ZMARCH_3D = 4,      /* threads march along z in registers (n0 % 4 != 0) */
+    MXP_SWEEP_ZMARCH_TMA_3D = 5   /* threads march along z, planes staged by TMA (n0 % 4 == 0) */
 } mxp_sweep_kind;
 /* With fuse_k = 0 the exp actions of the two z-marching kinds take two steps per
- * launch (planes staged by TMA, rows padded where n0 % 4 != 0); the results are those
- * of single steps to the last bit. */
+ * launch (planes staged by TMA, rows padded where n0 % 4 != 0) where the set-up times
+ * that as the faster form; the results are those of single steps to the last bit. */
 /* Returns an mxp_sweep_kind, or -1 for a NULL problem or a failed set-up.
  * For 3D low-precision problems it may allocate the problem's work buffers and
  * build their TMA descriptors (as the first action would). */

@@ -125,6 +125,7 @@ struct mxp_problem {
     double fused_cost = 1e30;  // estimated ms per exp action with the per-pass kernels
     int persist_cfg = -1;      // persistent exp-action kernel (2D), -1 = not used
     int f3_cfg = -1, f3_lz = 64;   // fused 3D exp sweeps, -1 = unfused
+    bool f3_two = true;            // unfused 3D exp actions take two steps per launch (fuse_k = 0)
     int p_txo = 0, p_tyo = 0, p_ntx = 0, p_nty = 0;
     float *tau_dev = nullptr;  // per-step tau / h^2 of the exp plan (persistent kernel)
     size_t tau_cap = 0;
@@ -732,13 +733,55 @@ static mxp_status tune_persist(mxp_problem *P, double best_cost)
     return MXP_OK;
 }
 
-// Pick the 3D exp sweep: time a few passes of each fused z-marching
-// configuration (and segment length) and the unfused kernel; keep the one with
-// the smallest (sweeps per action) x (time per sweep).  fuse_k as in 2D.
+// Whether the unfused 3D exp actions take two steps per launch (tma3d2.cu): unless
+// single steps are faster (tune_fused3) or asked for (fuse_k = 1).
+static bool tma3_two(const mxp_problem *P) { return P->prm.fuse_k == 0 && P->f3_two; }
+
+// Tensor maps for the TMA-staged 3D sweeps of this problem, or nullptr when the
+// grid or the driver does not allow them (the register-marching sweep is used).
+// Rows that are no multiple of 4 are padded for the two-step sweeps; single-step
+// sweeps and psi actions of such grids march in registers.
+template <typename S>
+static const Tma3Maps *tma3_maps(mxp_problem *P, bool padded)
+{
+    if (P->grid.dim != 3 || P->nfaces) return nullptr;
+    const int n0 = P->geom.n[0], pitch = tma3_pitch(P->geom);
+    if (pitch != n0 && (!padded || P->lean)) return nullptr;
+    const int64_t rows = (int64_t)P->geom.n[1] * P->geom.n[2];
+    if (pitch > n0 && !P->kappa_pad_ok) {
+        if (capturing(P->stream)) return nullptr;
+        if (!P->kappa_pad && cudaMalloc(&P->kappa_pad, (size_t)rows * pitch * sizeof(float)) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (cudaMemcpy2DAsync(P->kappa_pad, pitch * sizeof(float), P->kappa32, n0 * sizeof(float), n0 * sizeof(float),
+                              (size_t)rows, cudaMemcpyDeviceToDevice, P->stream) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        P->kappa_pad_ok = true;
+    }
+    if (P->tma3_prec == (int)P->prm.prec) return P->tma3;
+    tma3_destroy(P->tma3);
+    P->tma3 = tma3_create<S>(P->geom, P->hb, pitch > n0 ? P->kappa_pad : P->kappa32);
+    P->tma3_prec = (int)P->prm.prec;
+    return P->tma3;
+}
+
+// Pick the 3D exp sweep: time a few passes of each fused z-marching configuration (and
+// segment length) and of the unfused kernels, and keep what has the smallest (sweeps per
+// action) x (time per sweep).  The unfused candidates are those an action would run: two
+// steps per launch and single steps, staged by TMA where the rows allow it, else marching
+// in registers (the same values either way).  Two steps per launch win in complex64 (1.1
+// to 4.5 times) and on most bf16 grids, single steps on some bf16 ones (192^3: 69.1
+// against 69.9 ms an action, 160^3 44.5 and 45.0).  k_fused3d, which wins on the smallest
+// grids against single steps (60 x 28 x 3: 5.11 ms an action, two steps per launch 2.41),
+// was the fastest on none of 21 grids from 6 to 23.9 M unknowns.  fuse_k as in 2D.
 template <typename S>
 static mxp_status tune_fused3(mxp_problem *P)
 {
     P->f3_cfg = -1;
+    P->f3_two = true;
     if (P->grid.dim != 3 || P->prm.prec == MXP_C128 || P->prm.fuse_k == 1) return MXP_OK;
     if (P->prm.tile_cfg >= 0) {
         if (P->prm.tile_cfg >= fused3d_num_cfgs()) return fail(MXP_EINVAL, "tile_cfg out of range for 3D");
@@ -747,56 +790,78 @@ static mxp_status tune_fused3(mxp_problem *P)
         return MXP_OK;
     }
     CKS(ensure_base(P));
-    const int64_t n = P->ntot;
-    S *b0 = (S *)P->hb[0], *b1 = (S *)P->hb[1], *b2 = (S *)P->hb[2];
-    CK(cudaMemsetAsync(b0, 0, (size_t)n * sizeof(S), P->stream));
-    CK(cudaMemsetAsync(b1, 0, (size_t)n * sizeof(S), P->stream));
+    S *b[3] = {(S *)P->hb[0], (S *)P->hb[1], (S *)P->hb[2]};
+    const Tma3Maps *tm2 = P->prm.fuse_k == 0 ? tma3_maps<S>(P, true) : nullptr;
+    const int n0 = P->geom.n[0];
+    const size_t bytes = (size_t)(P->ntot / n0) * (tm2 ? tma3_maps_pitch(tm2) : n0) * sizeof(S);
+    CK(cudaMemsetAsync(b[0], 0, bytes, P->stream));
+    CK(cudaMemsetAsync(b[1], 0, bytes, P->stream));
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
+    StepScalars<typename St<S>::C> sc;
+    sc.zfac = PrecData<S>::c(cd(1.0, P->prm.shift_s));
+    sc.mu = 0;
+    sc.sigma = PrecData<S>::c(cd(0.0, 1e-9));
+    sc.gamma = PrecData<S>::c(cd(0.0));
+    sc.rho = PrecData<S>::c(cd(1.0));
+    mxp_status err = MXP_OK;
+    // ms per step of `passes` launches of K steps each, the best of two after a first
+    auto time_steps = [&](int passes, int K, auto launch) {
+        float best = 1e30f;
+        for (int rep = 0; rep < 3 && err == MXP_OK; ++rep) {
+            cudaEventRecord(e0, P->stream);
+            cudaError_t ce = cudaSuccess;
+            for (int i = 0; i < passes && ce == cudaSuccess; ++i) ce = launch((i & 1) ? 2 : 1, (i & 1) ? 1 : 2, i > 0);
+            cudaEventRecord(e1, P->stream);
+            if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
+            if (ce == cudaSuccess) ce = cudaGetLastError();
+            if (ce != cudaSuccess) err = fail(MXP_ECUDA, std::string("timing the 3D sweeps: ") + cudaGetErrorString(ce));
+            float ms = 0;
+            cudaEventElapsedTime(&ms, e0, e1);
+            if (rep > 0) best = std::min(best, ms);
+        }
+        return best / (passes * (double)K);
+    };
     double best = -1;
     int best_cfg = -1, best_lz = 64;
-    for (int cfg = -1; cfg < fused3d_num_cfgs(); ++cfg) {
-        const int K = cfg >= 0 ? fused3d_cfg_k(cfg) : 1;
-        if (P->prm.fuse_k > 1 && K != P->prm.fuse_k) continue;
+    auto consider = [&](int cfg, int lz, int K, double step_ms) {
         const TaylorPlan pl = make_plan(P->nu, P->prm.exp_tol, theta_of(P), K);
-        for (int lz : {32, 64, 128}) {
-            if (cfg < 0 && lz != 32) continue;
-            FusedStep steps[kMaxFuse];
-            for (int s = 0; s < K; ++s) steps[s] = FusedStep{1e-9, 0, 0, 1, 0, 0};
-            const int passes = std::max(2, 8 / K);
-            float best_ms = 1e30f;
-            for (int rep = 0; rep < 3; ++rep) {
-                cudaEventRecord(e0, P->stream);
-                for (int i = 0; i < passes; ++i) {
-                    if (cfg >= 0) {
-                        launch_fused3d<S>(cfg, lz, P->geom, P->coef32, P->kappa32, steps,
-                                          make_float2(1.0f, (float)P->prm.shift_s), (i & 1) ? b2 : b1, b0,
-                                          (i & 1) ? b1 : b2, P->stream);
-                    } else {
-                        StepScalars<typename St<S>::C> sc;
-                        sc.zfac = PrecData<S>::c(cd(1.0, P->prm.shift_s));
-                        sc.mu = 0;
-                        sc.sigma = PrecData<S>::c(cd(0.0, 1e-9));
-                        sc.gamma = PrecData<S>::c(cd(0.0));
-                        sc.rho = PrecData<S>::c(cd(1.0));
-                        launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc,
-                                       (i & 1) ? b2 : b1, b0, nullptr, (i & 1) ? b1 : b2, P->stream);
-                    }
-                }
-                cudaEventRecord(e1, P->stream);
-                CK(cudaEventSynchronize(e1));
-                CK(cudaGetLastError());
-                float ms = 0;
-                cudaEventElapsedTime(&ms, e0, e1);
-                if (rep > 0) best_ms = std::min(best_ms, ms);
-            }
-            const double cost = best_ms / (passes * (double)K) * pl.S * pl.m;
-            if (best < 0 || cost < best) { best = cost; best_cfg = cfg; best_lz = lz; }
-        }
+        const double cost = step_ms * pl.S * pl.m;
+        if (best < 0 || cost < best) { best = cost; best_cfg = cfg; best_lz = lz; }
+    };
+    if (P->prm.fuse_k == 0) {
+        const Tma3Maps *tm1 = tma3_maps<S>(P, false);
+        const double one = time_steps(16, 1, [&](int in, int out, bool) {
+            if (tm1)
+                return launch_step3z_tma<S>(P->geom, PrecData<S>::coef(P), sc, tm1, in, 0, -1, b[out], P->bar + 2, P->stream);
+            launch_step<S>(P->geom, PrecData<S>::coef(P), PrecData<S>::kappa(P), sc, b[in], b[0], nullptr, b[out], P->stream);
+            return cudaSuccess;
+        });
+        double two = 1e30;
+        if (tm2)
+            two = time_steps(8, 2, [&](int in, int out, bool chain) {
+                return launch_step3z2<S>(P->geom, PrecData<S>::coef(P), sc, sc, tm2, in, 0, b[out], P->bar + 2, P->stream,
+                                         chain);
+            });
+        P->f3_two = two <= one;
+        consider(-1, 64, 1, std::min(one, two));
+    }
+    for (int cfg = 0; cfg < fused3d_num_cfgs(); ++cfg) {
+        const int K = fused3d_cfg_k(cfg);
+        if (P->prm.fuse_k > 1 && K != P->prm.fuse_k) continue;
+        FusedStep steps[kMaxFuse];
+        for (int s = 0; s < K; ++s) steps[s] = FusedStep{1e-9, 0, 0, 1, 0, 0};
+        for (int lz : {32, 64, 128})
+            consider(cfg, lz, K, time_steps(std::max(2, 8 / K), K, [&](int in, int out, bool) {
+                launch_fused3d<S>(cfg, lz, P->geom, P->coef32, P->kappa32, steps,
+                                  make_float2(1.0f, (float)P->prm.shift_s), b[in], b[0], b[out], P->stream);
+                return cudaSuccess;
+            }));
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    CKS(err);
     P->f3_cfg = best_cfg;
     P->f3_lz = best_lz;
     return MXP_OK;
@@ -873,41 +938,6 @@ static mxp_status retune(mxp_problem *P)
     make_plans(P);
     if (P->persist_cfg >= 0) CKS(upload_tau(P));
     return MXP_OK;
-}
-
-// Whether the 3D exp actions take two steps per launch (tma3d2.cu): unless the
-// parameters ask for unfused sweeps (fuse_k = 1).
-static bool tma3_two(const mxp_problem *P) { return P->prm.fuse_k == 0; }
-
-// Tensor maps for the TMA-staged 3D sweeps of this problem, or nullptr when the
-// grid or the driver does not allow them (the register-marching sweep is used).
-// Rows that are no multiple of 4 are padded for the two-step sweeps; single-step
-// sweeps and psi actions of such grids march in registers.
-template <typename S>
-static const Tma3Maps *tma3_maps(mxp_problem *P, bool padded)
-{
-    if (P->grid.dim != 3 || P->nfaces) return nullptr;
-    const int n0 = P->geom.n[0], pitch = tma3_pitch(P->geom);
-    if (pitch != n0 && (!padded || P->lean)) return nullptr;
-    const int64_t rows = (int64_t)P->geom.n[1] * P->geom.n[2];
-    if (pitch > n0 && !P->kappa_pad_ok) {
-        if (capturing(P->stream)) return nullptr;
-        if (!P->kappa_pad && cudaMalloc(&P->kappa_pad, (size_t)rows * pitch * sizeof(float)) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        if (cudaMemcpy2DAsync(P->kappa_pad, pitch * sizeof(float), P->kappa32, n0 * sizeof(float), n0 * sizeof(float),
-                              (size_t)rows, cudaMemcpyDeviceToDevice, P->stream) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        P->kappa_pad_ok = true;
-    }
-    if (P->tma3_prec == (int)P->prm.prec) return P->tma3;
-    tma3_destroy(P->tma3);
-    P->tma3 = tma3_create<S>(P->geom, P->hb, pitch > n0 ? P->kappa_pad : P->kappa32);
-    P->tma3_prec = (int)P->prm.prec;
-    return P->tma3;
 }
 
 // Scalar part of the augmented matrix of a psi action (which = 1: psi_1, one
