@@ -162,13 +162,15 @@ __device__ __forceinline__ uint32_t pk(float lo, float hi)
 // Predicated loads, zero where the predicate is false, issued where they stand and
 // straight into their registers: written as conditions, the compiler moves the loaded
 // values when the branches join, and waits for them there.
+// Plain loads, not .nc: a chained kernel starts while its predecessor still writes what
+// it will read, and .nc is for memory that is read-only as long as the kernel runs.
 __device__ __forceinline__ void ld4(float *v, const float *p, bool ok)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %5, 0;\n\t"
         "mov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\tmov.f32 %2, 0f00000000;\n\tmov.f32 %3, 0f00000000;\n\t"
-        "@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+        "@p ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
         : "=&f"(v[0]), "=&f"(v[1]), "=&f"(v[2]), "=&f"(v[3])
         : "l"(p), "r"((int)ok));
 }
@@ -179,9 +181,16 @@ __device__ __forceinline__ void ld1(float &v, const float *p, bool ok)
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %2, 0;\n\t"
         "mov.f32 %0, 0f00000000;\n\t"
-        "@p ld.global.nc.f32 %0, [%1];\n\t}"
+        "@p ld.global.f32 %0, [%1];\n\t}"
         : "=&f"(v)
         : "l"(p), "r"((int)ok));
+}
+
+__device__ __forceinline__ float ldg_now(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
 }
 
 // Input values behind 8 output pixels of one input row: v[1 .. LEN], with the
@@ -641,12 +650,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
                     if (a.o.add) {
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            if (j < nc) ad[j] = __ldg(a.o.add + q0 + (int64_t)j * hw);
+                            if (j < nc) ad[j] = ldg_now(a.o.add + q0 + (int64_t)j * hw);
                     }
                     if (GRAD && a.o.mask) {
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            if (j < nc) mk[j] = __ldg(a.o.mask + q0 + (int64_t)j * hw);
+                            if (j < nc) mk[j] = ldg_now(a.o.mask + q0 + (int64_t)j * hw);
                     }
                 }
                 uint32_t d[16];
@@ -670,7 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
                     if (owner && a.o.mask) {
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            if (j < nc) mk[j] = __ldg(a.o.mask + q4 + j * hw4);
+                            if (j < nc) mk[j] = ldg_now(a.o.mask + q4 + j * hw4);
                     }
                     asm volatile("bar.sync 1, 128;" ::: "memory");
                     if (owner) {

@@ -19,3 +19,16 @@ def _source(name):
 def test_release_follows_the_wait(name):
     # one place in the source where a kernel waits, and the release right behind it
     assert re.findall(r"griddepcontrol\.(\w+)", _source(name)) == ["wait", "launch_dependents"]
+
+
+def _chained_sources():
+    return [f for f in sorted(os.listdir(CSRC)) if f.endswith(".cu") and "griddepcontrol.wait" in _source(f)]
+
+
+def test_no_read_only_loads_of_a_predecessors_output():
+    """A chained kernel runs while its predecessor writes its inputs: they must not be
+    read by loads for memory that is constant over the kernel's life (ld.global.nc,
+    __ldg).  Tables that no chained kernel writes are const __restrict__ arguments."""
+    assert len(_chained_sources()) == 3
+    for name in _chained_sources():
+        assert not re.findall(r"\.nc\b|__ldg\w*\s*\(", _source(name)), name
