@@ -132,6 +132,7 @@ struct mxp_cnn {
     float *gy = nullptr, *g5 = nullptr, *gh = nullptr, *gh2 = nullptr, *g1 = nullptr;
     double *partial = nullptr;
     unsigned *err = nullptr;       // set by a tensor-core convolution whose bounded wait gave up
+    float *part = nullptr;         // partial sums of the bias gradients, per layer and CTA
     float *loss_dev = nullptr;
     float *loss_host = nullptr;
     int adam_t = 0;
@@ -173,14 +174,14 @@ bool conv_bwd_data(const mxp_cnn *net, int l, const float *gout, int N, int Ho, 
                      net->err, net->stream, true);
 }
 
-// adds layer l's weight and bias gradients to net->g
+// adds layer l's weight gradient to net->g, and its bias gradient to those that sums adds
 bool conv_bwd_weight(const mxp_cnn *net, int l, const float *xin, int N, int Hs, int Ws, const float *gout, int Ho,
-                     int Wo)
+                     int Wo, BiasSums *sums)
 {
     const CnnLayer L = kNet[l];
     float *gw = net->g + layer_woff(l);
     return wgrad_tile(L.stride, L.ups, xin, N, L.cin, Hs, Ws, gout, L.cout, Ho, Wo, gw,
-                      gw + (int64_t)L.cin * L.cout * 9, net->err, net->stream, l < 5);
+                      gw + (int64_t)L.cin * L.cout * 9, net->part + l * bias_part_floats(), sums, net->err, net->stream, l < 5);
 }
 
 mxp_status check_shape(const mxp_cnn *net, int N, int H, int W)
@@ -214,38 +215,40 @@ mxp_status backward_impl(mxp_cnn *net, const float *x, const float *gy)
     cudaStream_t st = net->stream;
     CKC(cudaMemsetAsync(net->g, 0, net->np * sizeof(float), st));
     // layer 6; a5 = r5 + a1: its gradient goes on to a1 (g1) and, masked, to layer 5 (g5)
-    bool ok = conv_bwd_weight(net, 5, net->a[4], N, H, W, gy, H, W);
+    BiasSums sums;
+    bool ok = conv_bwd_weight(net, 5, net->a[4], N, H, W, gy, H, W, &sums);
     ConvOut o;
     o.out = net->g5;
     o.out2 = net->g1;
     o.mask = net->r5;
     ok = ok && conv_bwd_data(net, 5, gy, N, H, W, H, W, o);
     // layer 5: the gradient of up2(a4) is summed over 2 x 2 blocks
-    ok = ok && conv_bwd_weight(net, 4, net->a[3], N, H2, W2, net->g5, H, W);
+    ok = ok && conv_bwd_weight(net, 4, net->a[3], N, H2, W2, net->g5, H, W, &sums);
     o = ConvOut{};
     o.out = net->gh;
     o.mask = net->a[3];
     o.pool = 1;
     ok = ok && conv_bwd_data(net, 4, net->g5, N, H, W, H, W, o);
     // layer 4
-    ok = ok && conv_bwd_weight(net, 3, net->a[2], N, H2, W2, net->gh, H2, W2);
+    ok = ok && conv_bwd_weight(net, 3, net->a[2], N, H2, W2, net->gh, H2, W2, &sums);
     o = ConvOut{};
     o.out = net->gh2;
     o.mask = net->a[2];
     ok = ok && conv_bwd_data(net, 3, net->gh, N, H2, W2, H2, W2, o);
     // layer 3
-    ok = ok && conv_bwd_weight(net, 2, net->a[1], N, H2, W2, net->gh2, H2, W2);
+    ok = ok && conv_bwd_weight(net, 2, net->a[1], N, H2, W2, net->gh2, H2, W2, &sums);
     o.out = net->gh;
     o.mask = net->a[1];
     ok = ok && conv_bwd_data(net, 2, net->gh2, N, H2, W2, H2, W2, o);
     // layer 2 (stride 2), plus the skip's gradient
-    ok = ok && conv_bwd_weight(net, 1, net->a[0], N, H, W, net->gh, H2, W2);
+    ok = ok && conv_bwd_weight(net, 1, net->a[0], N, H, W, net->gh, H2, W2, &sums);
     o.out = net->g5;
     o.add = net->g1;
     o.mask = net->a[0];
     ok = ok && conv_bwd_data(net, 1, net->gh, N, H2, W2, H, W, o);
     // layer 1
-    ok = ok && conv_bwd_weight(net, 0, x, N, H, W, net->g5, H, W);
+    ok = ok && conv_bwd_weight(net, 0, x, N, H, W, net->g5, H, W, &sums);
+    ok = ok && launch_bias_sums(sums, st);
     if (!ok) return cfail(MXP_ECUDA, "launch of a convolution failed");
     CKC(cudaGetLastError());
     return MXP_OK;
@@ -289,6 +292,7 @@ mxp_status mxp_cnn_create(int device, void *cuda_stream, int max_batch, int max_
     A((void **)&net->gh, half * 64 * 4); A((void **)&net->gh2, half * 64 * 4);
     A((void **)&net->partial, 2048 * sizeof(double)); A((void **)&net->loss_dev, sizeof(float));
     A((void **)&net->err, sizeof(unsigned));
+    A((void **)&net->part, 6 * bias_part_floats() * sizeof(float));
     ok = ok && cudaMallocHost((void **)&net->loss_host, sizeof(float)) == cudaSuccess;
     if (ok) {
         ok = cudaMemsetAsync(net->w, 0, net->np * 4, net->stream) == cudaSuccess &&
@@ -406,6 +410,7 @@ void mxp_cnn_destroy(mxp_cnn *net)
     for (float *b : bufs) cudaFree(b);
     cudaFree(net->wb);
     cudaFree(net->err);
+    cudaFree(net->part);
     cudaFree(net->partial);
     if (net->loss_host) cudaFreeHost(net->loss_host);
     delete net;

@@ -465,7 +465,7 @@ static bool conv_wgrad_tc(int S, int UPS, const float *x, int N, int Cin, int Hs
     const dim3 grid((unsigned)((npix + kWgradSteps * 16 - 1) / (kWgradSteps * 16)), (unsigned)((K + 127) / 128));
     if (cudaMemsetAsync(gw, 0, (size_t)Cout * K * sizeof(float), st) != cudaSuccess) return false;
     if (conv_tile_fits(Cin, Cout))
-        return wgrad_tile(S, UPS, x, N, Cin, Hs, Ws, g, Cout, Ho, Wo, gw, nullptr, err, st);
+        return wgrad_tile(S, UPS, x, N, Cin, Hs, Ws, g, Cout, Ho, Wo, gw, nullptr, nullptr, nullptr, err, st);
     count_launch();
     if (S == 2 && !UPS) launch_wgrad<2, 0>(Cout, grid, st, x, Cin, Hs, Ws, g, Ho, Wo, npix, gw, err);
     else if (S == 1 && UPS) launch_wgrad<1, 1>(Cout, grid, st, x, Cin, Hs, Ws, g, Ho, Wo, npix, gw, err);

@@ -40,6 +40,7 @@
 // Every wait on an mbarrier is bounded; on timeout the kernel sets *err, all roles
 // leave their loops, the issuer waits (bounded) for its last commit, and the
 // tensor memory is freed.
+#include <algorithm>
 #include <cstdint>
 
 #include "mxp_internal.h"
@@ -733,14 +734,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
 // step.  A step holds every k row of 64 pixels (72 KB) and the gradients of the same
 // pixels; all accumulators stay in tensor memory over the CTA's pixel tiles and are
 // added to gW once at the end.  The producers read the gradient tiles anyway and sum
-// them for the bias gradient.
+// them for the bias gradient: each CTA leaves its sums, and k_bias_sum adds those of all
+// layers in the CTAs' order, so that the same inputs give the same bits (with atomicAdd
+// they did not; added up by the last CTA of each layer it cost 3 to 5 us a layer, in one
+// launch behind them all 2 to 4 us in all).
 struct WgradArgs {
     const float *x;
     int Cin, Hs, Ws;
     const float *g;
     int Cout, Ho, Wo;
     int vecg;
-    float *gw, *gb;          // gb nullable
+    float *gw, *part;        // part nullable: [CTA][kMaxCh] sums of g
     int ntx, nty, ntiles, NT, nmb;
     bool chain;
     unsigned *err;
@@ -853,11 +857,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
         } else {
             while (stage(q[0], q[2]) && stage(q[1], q[0]) && stage(q[2], q[1])) {}
         }
-        if (a.gb && !*abort) {
+        if (a.part) {
+            unsigned cta;        // read here: held since the kernel's start it costs a register in the loop
+            asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
 #pragma unroll
             for (int it = 0; it < 2; ++it) {
                 for (int o = 1; o < 8; o <<= 1) bsum[it] += __shfl_xor_sync(0xffffffffu, bsum[it], o);
-                if (gc == 0 && gco + 32 * it < a.Cout) atomicAdd(a.gb + gco + 32 * it, bsum[it]);
+                if (gc == 0) a.part[cta * kMaxCh + gco + 32 * it] = bsum[it];
             }
         }
     } else if (warp == 4) {
@@ -910,12 +916,40 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
     if (warp == 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tcols));
 }
 
+// One block per layer: gb[co] += sum over its CTAs of part[CTA][co].  It is a few loads'
+// latency behind the last layer, so a thread takes every sixteenth CTA: up to twelve
+// loads at once, added in order, then the sixteen sums in order.
+constexpr int kSumWays = 16, kSumLoads = 12;
+
+__global__ void __launch_bounds__(kSumWays * kMaxCh) k_bias_sum(const __grid_constant__ BiasSums b)
+{
+    __shared__ float sum[kSumWays][kMaxCh];
+    const BiasSums::Layer L = b.layer[blockIdx.x];
+    const int co = threadIdx.x % kMaxCh, q = threadIdx.x / kMaxCh;
+    float t = 0.f;
+    wait_for_previous();
+    for (int c0 = q; c0 < L.ctas; c0 += kSumWays * kSumLoads) {
+        float v[kSumLoads];
+#pragma unroll
+        for (int i = 0; i < kSumLoads; ++i)
+            ld1(v[i], L.part + (c0 + i * kSumWays) * kMaxCh + co, c0 + i * kSumWays < L.ctas);
+#pragma unroll
+        for (int i = 0; i < kSumLoads; ++i) t += v[i];
+    }
+    sum[q][co] = t;
+    __syncthreads();
+    if (q == 0 && co < L.Cout) {
+        for (int w = 1; w < kSumWays; ++w) t += sum[w][co];
+        L.gb[co] += t;
+    }
+}
+
 template <typename... P, typename A>
-bool launch_chained(void (*fn)(P...), unsigned grid, int smem, cudaStream_t st, bool chain, const A &a)
+bool launch_chained(void (*fn)(P...), unsigned grid, int smem, cudaStream_t st, bool chain, const A &a, int threads = kThreads)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at{};
@@ -1005,6 +1039,13 @@ int n_tile(int channels) { return channels <= 16 ? 16 : channels <= 32 ? 32 : 64
 
 }  // namespace
 
+size_t bias_part_floats() { return (size_t)sm_count() * kMaxCh; }
+
+bool launch_bias_sums(const BiasSums &b, cudaStream_t st)
+{
+    return launch_chained(k_bias_sum, b.n, 0, st, true, b, kSumWays * kMaxCh);
+}
+
 bool conv_tile_fits(int Cin, int Cout) { return Cin >= 1 && Cin <= kMaxCh && Cout >= 1 && Cout <= kMaxCh; }
 
 bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
@@ -1034,9 +1075,10 @@ bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int H
 }
 
 bool wgrad_tile(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
-                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st, bool chain)
+                int Wo, float *gw, float *gb, float *part, BiasSums *sums, unsigned *err, cudaStream_t st, bool chain)
 {
     WgradArgs a{};
+    a.part = part;
     a.chain = chain;
     a.x = x;
     a.Cin = Cin;
@@ -1048,12 +1090,12 @@ bool wgrad_tile(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, 
     a.Wo = Wo;
     a.vecg = aligned4(g, Wo);
     a.gw = gw;
-    a.gb = gb;
     a.NT = n_tile(Cout);
     a.nmb = (Cin * 9 + 127) / 128;
     a.err = err;
-    if (UPS) return launch_wgrad_w<kFU>(a, N, st);
-    return S == 2 ? launch_wgrad_w<kF2>(a, N, st) : launch_wgrad_w<kF1>(a, N, st);
+    const bool ok = UPS ? launch_wgrad_w<kFU>(a, N, st) : S == 2 ? launch_wgrad_w<kF2>(a, N, st) : launch_wgrad_w<kF1>(a, N, st);
+    if (ok && part) sums->layer[sums->n++] = {part, gb, std::min(a.ntiles, sm_count()), Cout};
+    return ok;
 }
 
 }  // namespace mxp

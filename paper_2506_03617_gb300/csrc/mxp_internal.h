@@ -339,9 +339,23 @@ bool conv_tile_fits(int Cin, int Cout);
 bool conv_tile(bool grad, int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
                const float *bias, int Cout, int Ho, int Wo, int relu, const ConvOut &o, unsigned *err, cudaStream_t st,
                bool chain = false);
-// Adds the weight gradient to gw (and the sums of g per channel to gb, nullable).
+// Adds the weight gradient to gw.  With part (bias_part_floats() floats, this layer's
+// own until the sums are made) it also leaves the sums of g per channel there and enters
+// them in sums; launch_bias_sums adds each entry to its gb, in an order that depends on
+// the sizes only (behind the last of these kernels on st, chained to it).
+struct BiasSums {
+    struct Layer {
+        const float *part;
+        float *gb;
+        int ctas, Cout;
+    } layer[8];
+    int n = 0;
+};
+size_t bias_part_floats();
 bool wgrad_tile(int S, int UPS, const float *x, int N, int Cin, int Hs, int Ws, const float *g, int Cout, int Ho,
-                int Wo, float *gw, float *gb, unsigned *err, cudaStream_t st, bool chain = false);
+                int Wo, float *gw, float *gb, float *part, BiasSums *sums, unsigned *err, cudaStream_t st,
+                bool chain = false);
+bool launch_bias_sums(const BiasSums &b, cudaStream_t st);
 
 // Learned stage: z = network(v) on a 2D grid (n0 x n1), see cnn.cu.
 mxp_status cnn_apply_vector(mxp_cnn *net, int n0, int n1, const double2 *v, double vnorm,
