@@ -37,9 +37,9 @@
 // of that batch, before these kernels 4.28 ms).  One forward pass on 1088^2: 0.68 ms,
 // before 2.98 ms.
 //
-// Every wait on an mbarrier is bounded; on timeout the kernel sets *err, all roles
-// leave their loops, the issuer waits (bounded) for its last commit, and the
-// tensor memory is freed.
+// Every wait on an mbarrier is bounded; on timeout the kernel sets *err, the issuer and
+// the epilogue leave their loops, the producers run to their end without waiting, the
+// issuer waits (bounded) for its last commit, and the tensor memory is freed.
 #include <algorithm>
 #include <cstdint>
 
@@ -73,7 +73,10 @@ __device__ __forceinline__ void bar_arrive(uint64_t *bar)
 }
 
 // Waits until the phase of the given parity has completed; false on timeout or
-// when another role gave up.
+// when another role gave up.  The lanes of a warp may differ in that, and must not part
+// over it in front of warp-wide instructions: the producers go on either way (to the end
+// of their tiles without waiting, into their own shared memory), the MMA issuer is one
+// lane, the epilogue warps vote.
 __device__ __forceinline__ bool bar_wait(uint64_t *bar, unsigned parity, volatile int *abort)
 {
     const uint32_t a = su32(bar);
@@ -551,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
             const TilePos p = at.pos(TH, TW);
             const int nch = min(kStageCh, a.Cin - at.s * kStageCh);
             // parity 1 of a fresh barrier counts as complete: the first round finds its slots free
-            if (!bar_wait(&sh.empty[slot], par, abort)) return false;
+            bar_wait(&sh.empty[slot], par, abort);
             uint8_t *base = sA + slot * 2 * kBlk;
             items.template store<false>(now, base, p, nch, a.Ho, a.Wo);
             const int k0 = nch * 9, k1 = (k0 + 15) / 16 * 16;
@@ -580,17 +583,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
         }
     } else if (warp == 4) {
         // ------------------------------------------------ MMA issuer
-        const uint32_t id = idesc_bf16(NT, 1);
-        bool ok = bar_wait(&sh.wready, 0, abort);
-        int n = 0, slot = 0, par = 0, last = -1, lastpar = 0;
-        for (int t = t0; ok && t < a.ntiles; t += dt, ++n) {
-            const int acc = n & 1;
-            if (n >= 2) ok = bar_wait(&sh.acc_empty[acc], ((n >> 1) - 1) & 1, abort);
-            for (int s = 0; ok && s < nst; ++s) {
-                ok = bar_wait(&sh.full[slot], par, abort);
-                if (!ok) break;
-                tc_after();
-                if (lane == 0) {
+        if (lane == 0) {
+            const uint32_t id = idesc_bf16(NT, 1);
+            bool ok = bar_wait(&sh.wready, 0, abort);
+            int n = 0, slot = 0, par = 0, last = -1, lastpar = 0;
+            for (int t = t0; ok && t < a.ntiles; t += dt, ++n) {
+                const int acc = n & 1;
+                if (n >= 2) ok = bar_wait(&sh.acc_empty[acc], ((n >> 1) - 1) & 1, abort);
+                for (int s = 0; ok && s < nst; ++s) {
+                    ok = bar_wait(&sh.full[slot], par, abort);
+                    if (!ok) break;
+                    tc_after();
                     // a lone warp runs at instruction latency: descriptors by addition, unrolled
                     // (36 MMAs of a tile took 111 cycles each with a loop that formed them)
                     const int nch = min(kStageCh, a.Cin - s * kStageCh);
@@ -606,21 +609,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
                     }
                     commit_to(&sh.empty[slot]);
                     if (s == nst - 1) commit_to(&sh.acc_full[acc]);
-                }
-                __syncwarp();
-                last = slot;
-                lastpar = par;
-                if (++slot == kSlots) {
-                    slot = 0;
-                    par ^= 1;
+                    last = slot;
+                    lastpar = par;
+                    if (++slot == kSlots) {
+                        slot = 0;
+                        par ^= 1;
+                    }
                 }
             }
+            // before the tensor memory is freed: every MMA issued has completed
+            if (last >= 0) {
+                volatile int none = 0;
+                bar_wait(&sh.empty[last], lastpar, &none);
+            }
         }
-        // before the tensor memory is freed: every MMA issued has completed
-        if (last >= 0) {
-            volatile int none = 0;
-            bar_wait(&sh.empty[last], lastpar, &none);
-        }
+        __syncwarp();
     } else {
         // ------------------------------------------------ weights, then epilogue
         load_weights(sB, a, GRAD, tid, 128);
@@ -827,7 +830,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
                         for (int e = 0; e < 8; ++e) ld1(gv[it][e], row + ox + e, ok && ox + e < a.Wo);
                     }
                 }
-                if (!bar_wait(&sh.empty[slot], par, abort)) return false;
+                bar_wait(&sh.empty[slot], par, abort);
             }
             items.template store<true>(now, base + gi * kStageK * 128, p, min(kStageCh, a.Cin - gi * kStageCh), a.Ho, a.Wo);
             if (gi == ngrp - 1) {
@@ -867,15 +870,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
             }
         }
     } else if (warp == 4) {
-        const uint32_t id = idesc_bf16(NT, 0);
-        bool ok = true;
-        int n = 0;
-        for (int t = t0; t < a.ntiles; t += dt, ++n) {
-            const int slot = n & 1;
-            ok = bar_wait(&sh.full[slot], (n >> 1) & 1, abort);
-            if (!ok) break;
-            tc_after();
-            if (lane == 0) {
+        if (lane == 0) {
+            const uint32_t id = idesc_bf16(NT, 0);
+            bool ok = true;
+            int n = 0;
+            for (int t = t0; t < a.ntiles; t += dt, ++n) {
+                const int slot = n & 1;
+                ok = bar_wait(&sh.full[slot], (n >> 1) & 1, abort);
+                if (!ok) break;
+                tc_after();
                 const uint32_t ab = su32(smem + slot * slotsz);
                 uint64_t ad = desc(ab, 16, 1024, 2);
                 const uint64_t bd = desc(ab + asz, 16, 1024, 2);
@@ -888,13 +891,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_wgrad_tile(const __grid_constan
                 commit_to(&sh.empty[slot]);
                 if (t + dt >= a.ntiles) commit_to(&sh.done);
             }
-            __syncwarp();
+            if (n > 0) {
+                volatile int none = 0;
+                bar_wait(&sh.empty[(n - 1) & 1], ((n - 1) >> 1) & 1, &none);
+            }
         }
-        if (n > 0) {
-            volatile int none = 0;
-            bar_wait(&sh.empty[(n - 1) & 1], ((n - 1) >> 1) & 1, &none);
-        }
-    } else if (bar_wait(&sh.done, 0, abort)) {
+        __syncwarp();
+    } else if (__all_sync(0xffffffffu, bar_wait(&sh.done, 0, abort))) {
         wait_for_previous();
         tc_after();
         for (int mb = 0; mb < a.nmb; ++mb) {
