@@ -400,12 +400,17 @@ static void launch_tc(int cout, dim3 grid, cudaStream_t st, const float *in, int
         k_conv_tc<MODE, S, UPS, 64><<<grid, 128, 0, st>>>(in, Cin, Hs, Ws, w, bias, cout, Ho, Wo, relu, out, npix, err);
 }
 
+// Layers for conv_tile.cu: all that it takes, except one channel spread over more than 32
+// (1 -> 64 channels on 32 x 64^2 pixels: 53 us a call there, 43 us here; 3 -> 64 53 and
+// 54).  That is stores only, for which its four epilogue warps an SM are too few.
+static bool tiled(int K, int N) { return conv_tile_fits(K, N) && !(K == 1 && N > 32); }
+
 static bool conv_fwd_tc(int S, int UPS, const float *in, int N, int Cin, int Hs, int Ws, const __nv_bfloat16 *w,
                         const float *bias, int Cout, int Ho, int Wo, int relu, float *out, unsigned *err,
                         cudaStream_t st)
 {
     if (Cout < 1 || Cout > 64 || Cin < 1 || (UPS && S != 1)) return false;
-    if (conv_tile_fits(Cin, Cout)) {
+    if (tiled(Cin, Cout)) {
         ConvOut o;
         o.out = out;
         return conv_tile(false, S, UPS, in, N, Cin, Hs, Ws, w, bias, Cout, Ho, Wo, relu, o, err, st);
@@ -424,7 +429,7 @@ static bool conv_bwd_data_tc(int S, const float *gout, int N, int Cout, int Ho, 
                              int Cin, int Hl, int Wl, float *gin, unsigned *err, cudaStream_t st)
 {
     if (Cin < 1 || Cin > 64 || Cout < 1) return false;
-    if (conv_tile_fits(Cout, Cin)) {
+    if (tiled(Cout, Cin)) {
         ConvOut o;
         o.out = gin;
         return conv_tile(true, S, 0, gout, N, Cout, Ho, Wo, w, nullptr, Cin, Hl, Wl, 0, o, err, st);
