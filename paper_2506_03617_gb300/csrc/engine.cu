@@ -165,34 +165,21 @@ struct mxp_problem {
 
 // ------------------------------------------------------------------ helpers
 
-static cd inv_stretch(const mxp_problem *P, int d, double x)
+static PmlAxis pml_axis(const mxp_problem *P, int d)
 {
-    const int p = P->grid.npml;
-    if (p == 0) return 1.0;
-    const double h = P->grid.h;
-    const double L = (double)P->grid.n_interior[d] * h;
-    const double delta = p * h;
-    double dist = 0.0;
-    if (x < 0.0) dist = -x;
-    if (x > L) dist = x - L;
-    const double r = dist / delta;
-    const cd s(1.0, P->prm.c_pml / (delta * P->prm.omega) * r * r);
-    return 1.0 / s;
+    return PmlAxis{P->grid.npml, P->grid.n_interior[d], P->grid.h, P->prm.c_pml, P->prm.omega};
 }
 
 static void build_coef_host(mxp_problem *P)
 {
     const int nm = P->geom.nmax;
-    const double h = P->grid.h, ih2 = 1.0 / (h * h);
     P->coef_host.assign((size_t)9 * nm, make_double2(0, 0));
     for (int d = 0; d < P->grid.dim; ++d) {
         const int64_t off = (P->slab && d == P->grid.dim - 1) ? P->row0 : 0;   // global index of local row 0
         for (int i = 0; i < P->geom.n[d]; ++i) {
-            const double x = ((double)(i + off) - P->grid.npml + 0.5) * h;
-            const cd a = inv_stretch(P, d, x);
-            const cd bp = inv_stretch(P, d, x + 0.5 * h);
-            const cd bm = inv_stretch(P, d, x - 0.5 * h);
-            const cd wp = a * bp * ih2, wm = a * bm * ih2, wc = wp + wm;
+            cd wp, wm;
+            pml_neighbours(pml_axis(P, d), i + off, false, &wp, &wm);
+            const cd wc = wp + wm;
             P->coef_host[(size_t)(3 * d + 0) * nm + i] = make_double2(wp.real(), wp.imag());
             P->coef_host[(size_t)(3 * d + 1) * nm + i] = make_double2(wm.real(), wm.imag());
             P->coef_host[(size_t)(3 * d + 2) * nm + i] = make_double2(wc.real(), wc.imag());
@@ -279,14 +266,12 @@ static void update_plans(mxp_problem *P)
     // per-axis coefficient classes (every PML index plus one interior index of
     // the whole grid, so that every slab of a grid gets the same plan)
     AxisClasses cls[3];
-    const double h = P->grid.h, ih2 = 1.0 / (h * h);
     for (int d = 0; d < P->grid.dim; ++d) {
         const int64_t n = P->grid.n_interior[d] + 2 * (int64_t)P->grid.npml, p = P->grid.npml;
         for (int64_t i = 0; i < n; ++i) {
             if (!(i < p || i >= n - p || i == p)) continue;
-            const double x = ((double)i - p + 0.5) * h;
-            const cd a = inv_stretch(P, d, x), bp = inv_stretch(P, d, x + 0.5 * h), bm = inv_stretch(P, d, x - 0.5 * h);
-            const cd wp = a * bp * ih2, wm = a * bm * ih2;
+            cd wp, wm;
+            pml_neighbours(pml_axis(P, d), i, true, &wp, &wm);
             cls[d].off.push_back(std::abs(wp) + std::abs(wm));
             cls[d].wc.push_back(wp + wm);
         }
@@ -324,10 +309,8 @@ static mxp_status upload_coef32(mxp_problem *P)
     return MXP_OK;
 }
 
-// The complex128 sweeps' table: coef_host times h^2.  Apart from upload_coefs so that
-// the compiler inlines and contracts build_coef_host there as it always has: other last
-// bits of the coefficients are differences of up to 5e-9 in a complex64 solve's solution.
-static __attribute__((noinline)) mxp_status upload_scaled64(mxp_problem *P)
+// The complex128 sweeps' table: coef_host times h^2.
+static mxp_status upload_scaled64(mxp_problem *P)
 {
     const double h2 = P->grid.h * P->grid.h;
     P->kappa_pad_ok = false;

@@ -33,6 +33,15 @@ struct TaylorPlan {
 // (S, m) minimising S*m with S (nu/S)^(m+1)/(m+1)! e^(nu/S) <= tol and
 // nu/S <= theta_max; m rounded up to a multiple of kmult.
 TaylorPlan make_plan(double nu, double tol, double theta_max, int kmult);
+// Neighbour coefficients wp, wm = a b+- / h^2 of grid position i of an axis (coef.cu);
+// bound: for the plan's row-sum bound, rounded in its own way.
+struct PmlAxis {
+    int npml;
+    int64_t n_interior;
+    double h, c_pml, omega;
+};
+void pml_neighbours(const PmlAxis &ax, int64_t i, bool bound, std::complex<double> *wp, std::complex<double> *wm);
+
 // Distinct coefficient classes of one axis: |wp| + |wm| and wc = wp + wm of
 // every PML position plus one interior position.
 struct AxisClasses {
