@@ -142,6 +142,7 @@ struct mxp_cnn {
 namespace {
 mxp_status cfail(mxp_status s, const char *m)
 {
+    if (s == MXP_ENOMEM || s == MXP_ECUDA) cudaGetLastError();      // as in engine.cu's fail
     mxp::note_error(m);
     return s;
 }

@@ -38,6 +38,9 @@ void mxp::note_error(const char *msg) { g_last_error = msg; }
 static mxp_status fail(mxp_status s, const std::string &msg)
 {
     g_last_error = msg;
+    // a failed call has reported the runtime's error: left there, the next call's check
+    // would find it and fail too
+    if (s == MXP_ENOMEM || s == MXP_ECUDA) cudaGetLastError();
     return s;
 }
 
