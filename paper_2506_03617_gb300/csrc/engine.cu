@@ -368,26 +368,38 @@ static void free_arnoldi(Arnoldi &a)
 
 static void clear_graphs(mxp_problem *P);
 
-// Device memory for vectors of the problem.  Where none is left, the tables that only
-// save time are given back and the sweeps do without them (the same results: diag_of
-// per point, the register-marching 3D sweep).
+// Gives back the tables that only save time: the scaled diagonal of the complex128
+// actions and (pad) the padded kappa of the low-precision 3D ones with its tensor maps.
+static void drop_tables(mxp_problem *P, bool diag, bool pad)
+{
+    if (!(diag && P->diag64) && !(pad && P->kappa_pad)) return;
+    cudaStreamSynchronize(P->stream);
+    clear_graphs(P);
+    if (diag) {
+        cudaFree(P->diag64);
+        P->diag64 = nullptr;
+        P->diag_ok = false;
+    }
+    if (pad && P->kappa_pad) {
+        tma3_destroy(P->tma3);
+        P->tma3 = nullptr;
+        P->tma3_prec = -1;
+        cudaFree(P->kappa_pad);
+        P->kappa_pad = nullptr;
+        P->kappa_pad_ok = false;
+    }
+}
+
+// Device memory for vectors of the problem.  Where none is left, the tables are given
+// back and the sweeps do without them until the parameters change (the same results:
+// diag_of per point, the register-marching 3D sweep).
 template <typename T>
 static cudaError_t dev_alloc(mxp_problem *P, T **p, size_t bytes)
 {
     const cudaError_t e = cudaMalloc((void **)p, bytes);
     if (e != cudaErrorMemoryAllocation || P->lean || (!P->diag64 && !P->kappa_pad)) return e;
     cudaGetLastError();
-    cudaStreamSynchronize(P->stream);
-    clear_graphs(P);
-    cudaFree(P->diag64);
-    P->diag64 = nullptr;
-    P->diag_ok = false;
-    if (P->kappa_pad) {
-        tma3_destroy(P->tma3);
-        P->tma3 = nullptr;
-        cudaFree(P->kappa_pad);
-        P->kappa_pad = nullptr;
-    }
+    drop_tables(P, true, true);
     P->lean = true;
     return cudaMalloc((void **)p, bytes);
 }
@@ -2566,6 +2578,7 @@ mxp_status mxp_set_boundary(mxp_problem *P, const int *bc)
     P->nfaces = nf;
     CKS(build_faces(P));
     P->diag_ok = false;
+    P->lean = false;
     clear_graphs(P);
     return retune(P);
 }
@@ -2609,6 +2622,8 @@ mxp_status mxp_set_params(mxp_problem *P, const mxp_params *p)
     update_plans(P);
     CKS(upload_coef32(P));
     P->diag_ok = false;
+    P->lean = false;
+    if (!P->slab) drop_tables(P, np.prec != MXP_C128, np.prec == MXP_C128);   // of the other type's actions
     if (P->slab) CKS(ensure_diag(P));
     clear_graphs(P);
     return retune(P);
@@ -2859,6 +2874,24 @@ mxp_status mxp_solve_batch(mxp_problem *const *probs, int nprob, int nrhs, const
             for (const mxp_solve_stats &q : stats[gi])
                 if (!q.converged) status[gi] = MXP_ENOCONV;
     };
+    // memory of the problems that run in threads, one after another: a problem's vectors
+    // may need what the others' tables take (a failure that stays is reported by its run)
+    for (size_t gi = 0; gi < ng; ++gi) {
+        mxp_problem *P = handles[gi];
+        if (in_group[gi] || coop[gi] || ng < 2 || P->prm.precond != 0) continue;
+        DeviceGuard guard(P->device);
+        auto memory = [&] {
+            const mxp_status s = ensure_base(P);
+            return s == MXP_OK ? ensure_batch(P, (int)groups[gi].size(), opts->restart, P->prm.inner_restart) : s;
+        };
+        if (memory() != MXP_ENOMEM) continue;
+        for (mxp_problem *Q : handles)
+            if (Q->device == P->device) {
+                drop_tables(Q, true, true);
+                Q->lean = true;
+            }
+        memory();
+    }
     // the group and the remaining problems run concurrently, one host thread
     // each (their kernels overlap on the GPU when they use different streams);
     // problems on the persistent kernel run afterwards, one at a time
