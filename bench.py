@@ -61,6 +61,27 @@ def alg_flops_per_update(grid):
     return (ALG_FLOPS_INTERIOR[grid.dim] * n_int + ALG_FLOPS_PML * (n - n_int)) / n
 
 
+# FP64 instructions of one complex128 update with y (a multiply-add takes the pipe as long
+# as an addition), by the number of axes in whose PML the cell lies
+FP64_INSTR = {2: (12, 16, 22), 3: (16, 20, 24, 30)}
+
+
+def fp64_instr_per_update(grid):
+    """FP64 instructions per point update of a complex128 sweep, over the grid's cells."""
+    cells = [1]                              # cells by number of PML axes, one axis after another
+    for ni in grid.ni:
+        inner, pml = int(ni), 2 * int(grid.npml)
+        cells = [(cells[k] * inner if k < len(cells) else 0) + (cells[k - 1] * pml if k else 0)
+                 for k in range(len(cells) + 1)]
+    return sum(c * i for c, i in zip(cells, FP64_INSTR[grid.dim])) / grid.n_total
+
+
+def sweep_bytes(prec, n, launches):
+    """Algorithmic bytes of `launches` passes over the vectors of n unknowns: a launch reads
+    p, y and kappa and writes p once, whether it takes one Taylor step or two."""
+    return BYTES_PER_PT[prec] * n * launches
+
+
 def nvtx_range(name):
     """Open (name) or close (None) an NVTX range, where torch has NVTX."""
     import torch
@@ -496,13 +517,14 @@ def run_ours(args):
             torch.cuda.synchronize()
             ev0 = torch.cuda.Event(enable_timing=True)
             ev1 = torch.cuda.Event(enable_timing=True)
+            nl3 = N.kernel_launch_count()
             ev0.record(P3.stream)
             ps3 = P3.apply_phi(0, x3, out=y3)[1]
             ev1.record(P3.stream)
             ev1.synchronize()
+        nl3 = N.kernel_launch_count() - nl3 - 2          # without the two conversions
         t3 = ev0.elapsed_time(ev1) / 1e3
-        sw3 = t3 / ps3
-        a3 = BYTES_PER_PT[args.prec] * g3.n_total / sw3 / 1e9
+        a3 = sweep_bytes(args.prec, g3.n_total, nl3) / t3 / 1e9
         # one whole MatExPre apply (psi_1 action, inner GMRES on exp actions, the
         # FP64 Krylov vectors) and one solve of the 288^3 point-source problem
         b3 = torch.from_numpy(I.rhs_from_source(I.gaussian_source(g3)).ravel()).to(f"cuda:{dev}")
@@ -515,19 +537,23 @@ def run_ours(args):
             ev1.record(P3.stream)
             ev1.synchronize()
         tm3 = ev0.elapsed_time(ev1) / 1e3
-        am3 = BYTES_PER_PT[args.prec] * g3.n_total * ast["stencil_passes"] / tm3 / 1e9
+        _, S1, m1 = P3.plan(1)                           # psi_1 in single steps, then exp actions
+        nx3 = (ast["stencil_passes"] - S1 * m1) / ps3
+        am3 = sweep_bytes(args.prec, g3.n_total, S1 * m1 + nx3 * nl3) / tm3 / 1e9
         row3 = _timed_solve(P3, b3, maxit=300)
         extra["hbm_resident_3d"] = {
             "workload": "3d_homogeneous_288 (256^3 + 16-cell PML)",
-            "exp_action": {"gpts": g3.n_total * ps3 / t3 / 1e9, "sweeps": ps3, "achieved_gbs": a3,
-                           "frac": a3 / peak},
+            "exp_action": {"gpts": g3.n_total * ps3 / t3 / 1e9, "sweeps": ps3, "launches": nl3,
+                           "achieved_gbs": a3, "frac": a3 / peak,
+                           "bound": "issue slots (two steps share a pass over memory)" if nl3 < ps3 else "hbm"},
             "matexpre_apply": {"seconds": tm3, "sweeps": ast["stencil_passes"],
                                "inner_iters": ast["inner_iters"],
                                "gpts": g3.n_total * ast["stencil_passes"] / tm3 / 1e9,
                                "sweep_bytes_gbs": am3, "frac": am3 / peak,
-                               "note": "sweep bytes (28 B per c64 point update) over the whole "
-                                       "apply's time, Krylov work included in the time"},
-            "solve": row3, "kernel": P3.sweep_kernel()}
+                               "note": "bytes of the sweeps' launches (28 B per c64 unknown and launch, of "
+                                       "one step or two) over the whole apply's time, Krylov work "
+                                       "included in the time"},
+            "solve": row3, "kernel": P3.sweep_kernel() + (", two steps per launch" if nl3 < ps3 else "")}
         del P3, x3, y3, b3, r3
         torch.cuda.empty_cache()
         # many sources per medium in lockstep (one sweep launch per pass for the batch)
@@ -573,6 +599,7 @@ def run_ours(args):
             t64 = ev0.elapsed_time(ev1) / 1e3
             pts64 = st64["pt_updates"]
             fl64 = alg_fpu * pts64 / t64 / 1e12
+            in64 = fp64_instr_per_update(grid) * pts64 / t64 / 1e12
             nrm64 = float(torch.linalg.vector_norm(x64))
             extra["fp64_solve"] = {"seconds": t64,
                                    "outer": st64["outer_iters"],
@@ -580,11 +607,14 @@ def run_ours(args):
                                    "true_relres": st64["true_relres"],
                                    "pt_updates": pts64, "gpts": pts64 / t64 / 1e9,
                                    "alg_tflops": fl64, "dfma_peak_tflops": fp64_peak,
-                                   "frac_of_dfma_peak": fl64 / fp64_peak,
+                                   "fp64_tera_instr": in64,
+                                   "frac_of_dfma_peak": in64 / (0.5 * fp64_peak),
                                    "roofline_note": "FP64 sweeps on an L2-resident grid: bound by "
-                                                    "the FP64 pipe (measured DFMA throughput, of measured); "
-                                                    "alg_tflops counts 24 flops per interior update, the "
-                                                    "sweep issues 12 FP64 instructions for them",
+                                                    "the FP64 pipe; the fraction is of its measured DFMA "
+                                                    "instruction rate and counts the sweeps' FP64 "
+                                                    "instructions (12 per interior update, which "
+                                                    "alg_tflops counts as 24 flops) over the whole "
+                                                    "solve's time",
                                    "speedup_of_this_precision": t64 / (total_max / args.steps),
                                    f"{args.prec}_solution_rel_err":
                                        float(torch.linalg.vector_norm(x_lo - x64)) / nrm64}
