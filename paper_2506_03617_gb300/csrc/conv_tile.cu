@@ -29,13 +29,12 @@
 // 5e-4 of the output.)
 //
 // What bounds it, measured by leaving parts out (64 -> 32 channels onto 1088^2 pixels,
-// 211 us, 206 TFLOP/s): the issue of the MMAs, 62 cycles each
-// whatever N is (135 us), under the stores of A (150 us without the loads); the loads'
-// latency adds 40 us, the epilogue 8 us.  The weights and the launch cost 12 us a
-// kernel, which is most of a layer on a batch of 32 crops of 64 x 64; as dependent
-// launches they run under the kernel before (0.57 -> 0.51 ms for forward and gradients
-// of that batch, before these kernels 4.28 ms).  One forward pass on 1088^2: 0.68 ms,
-// before 2.98 ms.
+// 200 us, 218 TFLOP/s; SM clock 2.07 GHz): the MMAs, 140 us for the 2196 of an SM, 130
+// cycles each; on top of them the stores of A 12 us, the epilogue 11 us, the loads'
+// latency 37 us.  The weights and the launch cost some 10 us a kernel, which is most of a
+// layer on a batch of 32 crops of 64 x 64; as dependent launches they run under the
+// kernel before (forward and gradients of that batch 0.50 ms, before these kernels
+// 4.28 ms).  One forward pass on 1088^2: 0.68 ms, before 2.98 ms.
 //
 // Every wait on an mbarrier is bounded; on timeout the kernel sets *err, the issuer and
 // the epilogue leave their loops, the producers run to their end without waiting, the
@@ -595,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_conv_tile(const __grid_constant
                     if (!ok) break;
                     tc_after();
                     // a lone warp runs at instruction latency: descriptors by addition, unrolled
-                    // (36 MMAs of a tile took 111 cycles each with a loop that formed them)
+                    // (with a loop that formed them the MMAs of a tile took 1.8 times as long)
                     const int nch = min(kStageCh, a.Cin - s * kStageCh);
                     const uint32_t dcol = tmem + acc * NT;
                     const uint64_t ad = desc(su32(sA + slot * 2 * kBlk), kBlk, 1024, 2);

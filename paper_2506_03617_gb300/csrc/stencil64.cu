@@ -4,15 +4,15 @@
 //
 // GB300 issues about two FP64 operations per clock and SM (1.05 TFLOP/s measured),
 // so an update costs what its FP64 instructions cost: the kernel is written for
-// their number, and memory (72 B per update, 2.2 TB/s at its rate) is far from a
-// bound.  Everything is scaled by h^2, so that a neighbour outside the PML has
-// coefficient 1 and costs an addition:
+// their number, and memory (64 B per update: p, y, the diagonal and the result;
+// 2.7 TB/s at its rate) is far from a bound.  Everything is scaled by h^2, so that a
+// neighbour outside the PML has coefficient 1 and costs an addition:
 //   q = sum_d (wp_d p_{+d} + wm_d p_{-d}) + D p,   D = h^2 (kappa (1 + i s) - mu - sum_d wc_d + faces),
 // with D read from a table that is made once per parameter set (k_diag64) and
 // sigma = i tau folded into two multiply-adds with y.  An interior 2D update is
 // then 6 additions + 4 + 2 multiply-adds = 12 FP64 instructions (3D: 16), where
 // the general form needs 32 (3D: 42); an axis in its PML adds 4 to 6.
-// Measured: 28.0 us a sweep of 1088^2 unknowns (42 G updates/s; 12 instructions at
+// Measured: 28.2 us a sweep of 1088^2 unknowns (42 G updates/s; 12 instructions at
 // the measured 0.527 T/s would be 27 us), the general form 117 us; 2.4 us a sweep of
 // 160^2, before 8.2 us; the psi_1 action on 128^3 127 ms, before 477 ms.
 #include "mxp_internal.h"
